@@ -346,7 +346,7 @@ typedef struct {
  *   - All calls on a device share the one scratch array.  Nothing in it needs clearing (every record a
  *     call reads, it has written first), but two calls whose kernels overlap on the GPU -- different
  *     streams, or the same image from two threads -- race on it: serialise them.
- *   - Enqueues two kernels on `stream` and returns without synchronising.
+ *   - Enqueues one or two kernels on `stream` and returns without synchronising.
  */
 lq_status_t lq_decode_attn_image_static(const lq_device_image_t* image, const void* q, float sm_scale,
                                         float* out, void* stream);

@@ -63,6 +63,51 @@ def test_static_scratch_entry_point_matches_the_cache_entry_point_and_the_oracle
         assert err <= attn_tolerance(other), ("lq_decode_attn", call, err)
 
 
+# (query heads per KV head, G, bits, n_fp, n_quant, elements by which every array starts off its 16-byte boundary, factor
+# on the value scales): every head count, no and ragged bf16 rows, one tile of a key group of 64 per warp, one split and
+# many, arrays that the wide copies cannot take, and scales near the end of the range
+FORMS = [(1, 32, 2, 0, 32, 0, 1.0), (1, 64, 4, 9, 64 * 31, 0, 1.0), (2, 32, 2, 1, 32 * 40, 0, 1.0), (2, 64, 2, 384, 0, 0, 1.0),
+         (3, 64, 2, 7, 64, 1, 1.0), (3, 32, 4, 63, 32 * 77, 0, 2.0 ** 118), (4, 32, 2, 385, 32 * 300, 0, 2.0 ** 119),
+         (4, 32, 4, 8, 32 * 33, 3, 1.0), (5, 64, 2, 127, 64 * 21, 0, 1.0), (6, 32, 2, 15, 32 * 2, 5, 1.0),
+         (7, 64, 4, 770, 64 * 130, 0, 1.0), (8, 32, 2, 16, 32 * 95, 0, 1.0), (8, 64, 2, 0, 64 * 9, 1, 1.0)]
+
+
+@pytest.mark.parametrize("r,G,bits,n_fp,n_quant,off,factor", FORMS)
+def test_random_images_against_the_same_attention_in_64_bits(r, G, bits, n_fp, n_quant, off, factor):
+    """Sums of up to 10^4 fp32 terms of either sign: 2^-24 times a few of them against the root of their sum of squares,
+    2e-6 seen; 1e-5 allowed."""
+    build.build()
+    B, H, gen = 3, 2, torch.Generator(device="cuda").manual_seed(r * 1000 + n_quant)
+
+    def place(x):  # a copy of x that starts `off` elements behind a 16-byte boundary
+        buf = torch.empty(x.numel() + 16, dtype=x.dtype, device="cuda")
+        y = buf[off:off + x.numel()].view(x.shape)
+        y.copy_(x)
+        return y
+
+    def normal(*shape):
+        return torch.randn(*shape, generator=gen, device="cuda", dtype=torch.bfloat16)
+
+    codes = [torch.randint(0, 256, (B, H, n_quant, D * bits // 8), generator=gen, device="cuda", dtype=torch.uint8)
+             for _ in range(2)]
+    top = 2 ** bits - 1
+    ks, vs = normal(B, H, n_quant // G, D).abs() / top, normal(B, H, n_quant, D // G).abs() / top * factor
+    kz, vz = normal(B, H, n_quant // G, D) - top / 2 * ks, normal(B, H, n_quant, D // G) * factor - top / 2 * vs
+    fp = [normal(B, H, n_fp, D), normal(B, H, n_fp, D) * factor]
+    q = normal(B, H * r, D)
+    arrays = dict(fp_k=fp[0], fp_v=fp[1], k_codes=codes[0], v_codes=codes[1], k_scale=ks, k_zero=kz, v_scale=vs, v_zero=vz)
+    image = {n: place(x if x.dtype == torch.uint8 else x.view(torch.int16)) for n, x in arrays.items()}
+    out = torch.full((B, H * r, D), float("nan"), device="cuda")
+    assert decode_attn_image_static(image, H * r, G, place(q), out, bits=bits) == binding.LQ_OK
+    code = [torch.stack([(c >> (bits * i)) & top for i in range(8 // bits)], dim=-1).flatten(3).double() for c in codes]
+    keys = kz.double().repeat_interleave(G, 2) + code[0] * ks.double().repeat_interleave(G, 2)
+    values = vz.double().repeat_interleave(G, 3) + code[1] * vs.double().repeat_interleave(G, 3)
+    keys, values = torch.cat([fp[0].double(), keys], 2), torch.cat([fp[1].double(), values], 2)
+    s = q.double().view(B, H, r, D) @ keys.transpose(2, 3) / np.sqrt(D)
+    want = (torch.softmax(s, 3) @ values).view(B, H * r, D)
+    assert float((out.double() - want).norm() / want.norm()) < 1e-5
+
+
 def _empty_image(B):
     z16 = torch.zeros(1, dtype=torch.int16, device="cuda")
     return dict(fp_k=torch.zeros(B, 1, 1, 128, dtype=torch.int16, device="cuda"),
