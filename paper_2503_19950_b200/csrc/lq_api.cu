@@ -757,7 +757,7 @@ lq_status_t ingest_prompt(lq_cache* c, int layer, const void* k, const void* v, 
   // pageable source: the runtime stages it before the call returns, so `idx` may die here
   cudaError_t e = cudaMemcpyAsync(c->ingest_idx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_fail(c, e, "prompt index upload");
-  e = launch_ingest(c->cv, layer, k, v, n, c->ingest_idx, n_tiles, has_fill, n_copy, tile0, st);
+  e = launch_ingest(c->cv, layer, k, v, n, c->ingest_idx, n_tiles, has_fill, n_copy, tile0, c->sm_count, st);
   if (e != cudaSuccess) return cuda_fail(c, e, "lq_ingest_kernel");
   { c->n_launches++; c->last_decode_layer = -1; }
   return LQ_OK;
