@@ -113,20 +113,42 @@ def exported_symbols():
 
 def _ptr(x):
     """Device/host address of a torch tensor, numpy array, int or None."""
-    if x is None:
-        return None
-    if isinstance(x, int):
-        return x
-    if isinstance(x, np.ndarray):
-        return x.ctypes.data
-    return x.data_ptr()  # torch tensor
+    try:
+        return x.data_ptr()  # torch tensor
+    except AttributeError:
+        return x.ctypes.data if isinstance(x, np.ndarray) else x
+
+
+_raw_stream = None  # torch's lookups of the current device and of its current stream's handle (one C call each)
 
 
 def _stream(stream):
+    """Handle of a stream (an int, a torch stream, or None: torch's current stream on the current device)."""
+    global _raw_stream
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream[1](_raw_stream[0]())
         import torch
-        return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else None
+        if not torch.cuda.is_available():
+            return None
+        handle = torch.cuda.current_stream().cuda_stream  # (initialises CUDA; the calls below do not)
+        _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+        return handle
     return stream if isinstance(stream, int) else stream.cuda_stream
+
+
+_bfloat16 = None
+
+
+def _out_dtype(out):
+    global _bfloat16
+    if _bfloat16 is None:
+        import torch
+        _bfloat16 = torch.bfloat16
+    return 1 if out.dtype == _bfloat16 else 0
+
+
+_IMAGE_ARRAYS = ("fp_k", "fp_v", "k_codes", "v_codes", "k_scale", "k_zero", "v_scale", "v_zero")
 
 
 def decode_attn_image_static(image: dict, n_q_heads: int, group: int, q, out, sm_scale=0.0, stream=None,
@@ -136,9 +158,8 @@ def decode_attn_image_static(image: dict, n_q_heads: int, group: int, q, out, sm
     B, Hkv, n_fp, D = image["fp_k"].shape
     n_quant = image["k_codes"].shape[2]
     st = lq_device_image_t(B, n_q_heads, Hkv, D, group, bits, n_fp, n_quant,
-                           *[(_ptr(image[k]) if image[k].numel() else None)
-                             for k in ("fp_k", "fp_v", "k_codes", "v_codes", "k_scale", "k_zero", "v_scale", "v_zero")])
-    return load_library().lq_decode_attn_image_static(C.byref(st), _ptr(q), sm_scale, _ptr(out), _stream(stream))
+                           *[(x.data_ptr() if x.numel() else None) for x in map(image.__getitem__, _IMAGE_ARRAYS)])
+    return (_lib or load_library()).lq_decode_attn_image_static(st, _ptr(q), sm_scale, _ptr(out), _stream(stream))
 
 
 class LogQuantCache:
@@ -153,6 +174,9 @@ class LogQuantCache:
         torch's caching allocator, kept alive until the cache is closed), or a pair of callables
         (alloc(bytes) -> device address or 0, free(address))."""
         self._lib = load_library()
+        # the calls of a decode step, bound once
+        self._append_decode_attn, self._decode_attn = self._lib.lq_append_decode_attn, self._lib.lq_decode_attn
+        self._decode_step_host = self._lib.lq_decode_step_host
         self._blocks = {}
         LogQuantCache.live.add(self)
         alloc_cb, free_cb = ALLOC_FN(0), FREE_FN(0)
@@ -214,22 +238,19 @@ class LogQuantCache:
 
     def append_decode_attn(self, layer, k, v, q, out, sm_scale=0.0, stream=None):
         """Append one token and run decode attention in one launch (k, v: [B, Hkv, 1, D] bf16)."""
-        import torch
         assert k.shape[2] == 1 and v.shape == k.shape
-        out_dtype = 1 if out.dtype == torch.bfloat16 else 0
-        self._check(self._lib.lq_append_decode_attn(self._h, layer, _ptr(k), _ptr(v), _ptr(q), sm_scale, _ptr(out),
-                                                    out_dtype, _stream(stream)))
+        status = self._append_decode_attn(self._h, layer, _ptr(k), _ptr(v), _ptr(q), sm_scale, _ptr(out), _out_dtype(out),
+                                          _stream(stream))
+        if status:
+            self._check(status)
 
     def decode_attn(self, layer, q, out, sm_scale=0.0, stream=None):
-        import torch
-        out_dtype = 1 if out.dtype == torch.bfloat16 else 0
-        self._check(self._lib.lq_decode_attn(self._h, layer, _ptr(q), sm_scale, _ptr(out), out_dtype,
-                                             _stream(stream)))
+        status = self._decode_attn(self._h, layer, _ptr(q), sm_scale, _ptr(out), _out_dtype(out), _stream(stream))
+        if status:
+            self._check(status)
 
     def decode_attn_fp_only(self, layer, q, out, sm_scale=0.0, stream=None):
-        import torch
-        out_dtype = 1 if out.dtype == torch.bfloat16 else 0
-        self._check(self._lib.lq_decode_attn_fp_only(self._h, layer, _ptr(q), sm_scale, _ptr(out), out_dtype,
+        self._check(self._lib.lq_decode_attn_fp_only(self._h, layer, _ptr(q), sm_scale, _ptr(out), _out_dtype(out),
                                                      _stream(stream)))
 
     def set_padding(self, pad):
@@ -244,8 +265,10 @@ class LogQuantCache:
         self._check(self._lib.lq_set_padding(self._h, C.cast(arr, C.c_void_p)))
 
     def decode_step_host(self, layer, k_host, v_host, q_host, out_host, sm_scale=0.0, sync=True, stream=None):
-        self._check(self._lib.lq_decode_step_host(self._h, layer, _ptr(k_host), _ptr(v_host), _ptr(q_host),
-                                                  sm_scale, _ptr(out_host), int(sync), _stream(stream)))
+        status = self._decode_step_host(self._h, layer, _ptr(k_host), _ptr(v_host), _ptr(q_host), sm_scale, _ptr(out_host),
+                                        int(sync), _stream(stream))
+        if status:
+            self._check(status)
 
     def profile_enable(self, on=True):
         self._check(self._lib.lq_profile_enable(self._h, int(on)))

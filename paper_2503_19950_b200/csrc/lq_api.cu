@@ -32,6 +32,20 @@ struct LayerState {
   std::vector<int32_t> quant_ids;   // token ids in 2-bit store order
 };
 
+// What an ingestion does to a layer depends on the layer's bookkeeping and the number of new tokens alone, and the layers of a
+// model are usually in the same state: the plan of one serves the others, index lists in device memory included.
+struct IngestPlan {
+  int n = 0;
+  LayerState before, after;  // (quant_ids left out)
+  std::vector<int32_t> ids;  // tokens that enter the 2-bit store, in store order
+  int n_tiles = 0, n_copy = 0;
+  bool has_fill = false;
+  int64_t idx_at = 0, idx_ints = 0;      // place in ingest_idx
+  unsigned long long uploaded_on = 0;    // id of the stream the lists were uploaded on (valid with `uploaded`)
+  bool uploaded = false;
+};
+constexpr int kMaxIngestPlans = 32;  // chunks of a prompt; more and they are made again for every layer
+
 }  // namespace
 
 struct lq_cache {
@@ -45,7 +59,9 @@ struct lq_cache {
   float* part_o = nullptr;
   float* part_ml = nullptr;
   int* status = nullptr;
-  int* ingest_idx = nullptr;  // index lists of the one-launch ingestion (3 max_tokens + 16 W + 3 G ints)
+  int* ingest_idx = nullptr;  // index lists of the one-launch ingestion (ingest_idx_ints)
+  std::vector<IngestPlan> plans;
+  int64_t idx_used = 0;       // ints of ingest_idx that belong to plans
   int* tickets = nullptr;  // per (b, kv) arrival counters of the fused split-K merge
   float* acc = nullptr;    // per (b, kv) sums of the partials added on arrival (DecodeArgs::acc)
   // staging for the host-buffer entry point, one slice per layer
@@ -101,12 +117,10 @@ lq_status_t cuda_fail(lq_cache* c, cudaError_t e, const char* what) {
   return LQ_ERR_CUDA;
 }
 
-constexpr int kGuardBytes = 256;       // after every device block; checked by lq_check_guards
-constexpr int kGuardPattern = 0xA5;
-
 // Every device block of a cache -- long-lived or temporary -- comes from here: the caller's allocator when one
 // is set, else cudaMalloc.  `bytes` is rounded up to 256 so that the guard starts on an aligned address.
-bool dev_alloc(lq_cache* c, void** p, int64_t bytes, bool temporary = false) {
+// guard = false: the caller fills the guard bytes in (launch_init_blocks).
+bool dev_alloc(lq_cache* c, void** p, int64_t bytes, bool temporary = false, bool guard = true) {
   const int64_t payload = (bytes + 255) / 256 * 256, total = payload + kGuardBytes;
   if (c->cfg.dev_alloc) {  // the caller's allocator
     *p = c->cfg.dev_alloc(static_cast<size_t>(total), c->cfg.alloc_ctx);
@@ -116,7 +130,7 @@ bool dev_alloc(lq_cache* c, void** p, int64_t bytes, bool temporary = false) {
     *p = nullptr;
     return false;
   }
-  if (cudaMemset(static_cast<uint8_t*>(*p) + payload, kGuardPattern, kGuardBytes) != cudaSuccess) cudaGetLastError();
+  if (guard && cudaMemset(static_cast<uint8_t*>(*p) + payload, kGuardPattern, kGuardBytes) != cudaSuccess) cudaGetLastError();
   c->blocks.emplace_back(static_cast<uint8_t*>(*p), payload);
   if (!temporary) c->bytes_device += total;
   return true;
@@ -161,6 +175,11 @@ void free_all(lq_cache* c) {
     dev_release(c, c->masks);
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   }
+}
+
+// ints of ingest_idx: up to three lists over the tokens that enter the 2-bit store and a copy list per plan
+int64_t ingest_idx_ints(const lq_cache* c) {
+  return 3 * (c->cfg.max_tokens + 3 * c->cfg.window + c->cfg.group) + kMaxIngestPlans * 2LL * (3 * c->cfg.window + c->cfg.group);
 }
 
 int ratio(const lq_cache* c) { return c->cfg.n_q_heads / c->cfg.n_kv_heads; }
@@ -479,8 +498,8 @@ lq_status_t lq_cache_create(const lq_config_t* cfg, lq_cache_t** out) {
   if (!c->dry) {
     cudaError_t e = cudaSetDevice(cfg->device);
     if (e != cudaSuccess) { delete c; cudaGetLastError(); return LQ_ERR_CUDA; }
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, cfg->device) == cudaSuccess) c->sm_count = prop.multiProcessorCount;
+    int sm_count = 0;  // (the whole property record takes 2.6 ms to fetch)
+    if (cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, cfg->device) == cudaSuccess) c->sm_count = sm_count;
     // split-K partial records reserved per (b, kv) (one more than the CTAs per pair: some pairs get an extra CTA)
     c->max_splits = 1 + (cfg->n_splits > 0
                         ? cfg->n_splits
@@ -488,24 +507,28 @@ lq_status_t lq_cache_create(const lq_config_t* cfg, lq_cache_t** out) {
     if (cfg->kernel == LQ_KERNEL_UMMA)  // the tcgen05 kernel cuts one cost line over all pairs: a few more slots per pair
       c->max_splits = std::max(c->max_splits, static_cast<int>(std::min<int64_t>(128, (2LL * c->sm_count + pairs - 1) / pairs + 3)));
     const int r = ratio(c);
-    bool ok = dev_alloc(c, reinterpret_cast<void**>(&cv.quant), cv.quant_layer_stride * cfg->n_layers) &&
-              dev_alloc(c, reinterpret_cast<void**>(&cv.fp), cv.fp_layer_stride * cfg->n_layers) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->part_o), pairs * c->max_splits * r * kD * 4) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->part_ml), pairs * c->max_splits * r * 2 * 4) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->status), 256) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->tickets), pairs * 128) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->acc), static_cast<int64_t>(pairs) * kAccStride * 4) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->ingest_idx), (3 * cfg->max_tokens + 16 * cfg->window + 3 * cfg->group) * 4) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->stage_k), cfg->n_layers * pairs * kD * 2) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->stage_v), cfg->n_layers * pairs * kD * 2) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->stage_q),
-                        static_cast<int64_t>(cfg->n_layers) * cfg->batch * cfg->n_q_heads * kD * 2) &&
-              dev_alloc(c, reinterpret_cast<void**>(&c->stage_out),
-                        static_cast<int64_t>(cfg->n_layers) * cfg->batch * cfg->n_q_heads * kD * 4);
-    if (ok) ok = cudaMemset(c->status, 0, 256) == cudaSuccess;
+    const int64_t q_bytes = static_cast<int64_t>(cfg->n_layers) * cfg->batch * cfg->n_q_heads * kD * 2;
+    const int64_t acc_bytes = static_cast<int64_t>(pairs) * kAccStride * 4;
+    auto alloc = [&](auto** p, int64_t bytes) { return dev_alloc(c, reinterpret_cast<void**>(p), bytes, false, false); };
+    bool ok = alloc(&cv.quant, cv.quant_layer_stride * cfg->n_layers) && alloc(&cv.fp, cv.fp_layer_stride * cfg->n_layers) &&
+              alloc(&c->part_o, pairs * c->max_splits * r * kD * 4) && alloc(&c->part_ml, pairs * c->max_splits * r * 2 * 4) &&
+              alloc(&c->status, 256) && alloc(&c->tickets, pairs * 128) && alloc(&c->acc, acc_bytes) &&
+              alloc(&c->ingest_idx, ingest_idx_ints(c) * 4) && alloc(&c->stage_k, cfg->n_layers * pairs * kD * 2) &&
+              alloc(&c->stage_v, cfg->n_layers * pairs * kD * 2) && alloc(&c->stage_q, q_bytes) && alloc(&c->stage_out, 2 * q_bytes);
     cv.status = c->status;
-    if (ok) ok = cudaMemset(c->tickets, 0, pairs * 128) == cudaSuccess;
-    if (ok) ok = cudaMemset(c->acc, 0, static_cast<size_t>(pairs) * kAccStride * 4) == cudaSuccess;
+    if (ok) {
+      BlockInit init;
+      std::memset(&init, 0, sizeof init);
+      for (const auto& blk : c->blocks) init.guard[init.n_guards++] = blk.first + blk.second;
+      auto zero = [&](void* p, int64_t bytes) {
+        init.zero[init.n_zero] = static_cast<uint4*>(p);
+        init.zero_chunks[init.n_zero++] = bytes / 16;
+      };
+      zero(c->status, 256);
+      zero(c->tickets, pairs * 128);
+      zero(c->acc, acc_bytes);
+      ok = launch_init_blocks(init, nullptr) == cudaSuccess;
+    }
     // the fp store must never hold non-finite garbage in unused slots of a partly filled tile
     if (ok) ok = cudaMemset(cv.fp, 0, static_cast<size_t>(cv.fp_layer_stride) * cfg->n_layers) == cudaSuccess;
     if (!ok) {
@@ -638,13 +661,63 @@ bool ingest_plan_is_sound(const LayerState& L, int W, bool top_in_place, const s
   return L.pend_slot.size() + L.age_slot.size() == static_cast<size_t>(L.n_fp);
 }
 
+bool same_bookkeeping(const LayerState& a, const LayerState& b) {
+  return a.n_seen == b.n_seen && a.n_quant == b.n_quant && a.n_fp == b.n_fp && a.n_events == b.n_events &&
+         a.age_slot == b.age_slot && a.pend_slot == b.pend_slot && a.slot_token == b.slot_token;
+}
+void copy_bookkeeping(LayerState& to, const LayerState& from) {  // all but quant_ids
+  to.n_seen = from.n_seen; to.n_events = from.n_events; to.n_quant = from.n_quant; to.n_fp = from.n_fp;
+  to.age_slot = from.age_slot; to.pend_slot = from.pend_slot; to.slot_token = from.slot_token;
+}
+
+// Index lists of a plan on the device, ready for a kernel on `st`.  Lists uploaded on this very stream are there already;
+// a stream that is being captured neither finds nor leaves any (its copy runs when the graph does).
+lq_status_t launch_plan(lq_cache* c, int layer, IngestPlan& p, const int32_t* idx, const void* k, const void* v, cudaStream_t st) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || cudaStreamGetId(st, &id) != cudaSuccess) {
+    cudaGetLastError();
+    capture = cudaStreamCaptureStatusActive;
+  }
+  const bool plain = capture == cudaStreamCaptureStatusNone;
+  cudaError_t e;
+  if (!(plain && p.uploaded && p.uploaded_on == id)) {
+    if (!idx) return LQ_ERR_UNSUPPORTED;  // (the caller makes the lists again)
+    // pageable source: the runtime stages it before the call returns, so `idx` may die here
+    e = cudaMemcpyAsync(c->ingest_idx + p.idx_at, idx, p.idx_ints * sizeof(int32_t), cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return cuda_fail(c, e, "prompt index upload");
+    p.uploaded = plain;
+    p.uploaded_on = id;
+  }
+  e = launch_ingest(c->cv, layer, k, v, p.n, c->ingest_idx + p.idx_at, p.n_tiles, p.has_fill, p.n_copy,
+                    p.before.n_quant / c->cfg.group, c->sm_count, st);
+  if (e != cudaSuccess) return cuda_fail(c, e, "lq_ingest_kernel");
+  { c->n_launches++; c->last_decode_layer = -1; }
+  return LQ_OK;
+}
+
 lq_status_t ingest_prompt(lq_cache* c, int layer, const void* k, const void* v, int n, cudaStream_t st) {
   LayerState& L = c->layers[layer];
   if (!c->mask_dirty.empty()) c->mask_dirty[layer] = 1;
+  for (IngestPlan& p : c->plans) {
+    if (p.n != n || !same_bookkeeping(p.before, L)) continue;
+    const lq_status_t s = launch_plan(c, layer, p, nullptr, k, v, st);
+    if (s == LQ_ERR_UNSUPPORTED) {  // its lists are on another stream
+      c->plans.clear();
+      c->idx_used = 0;
+      break;
+    }
+    copy_bookkeeping(L, p.after);
+    L.quant_ids.insert(L.quant_ids.end(), p.ids.begin(), p.ids.end());
+    return s;
+  }
+  IngestPlan plan;
+  plan.n = n;
+  copy_bookkeeping(plan.before, L);
   const int W = c->cfg.window, G = c->cfg.group;
   // the layer as it is now: token -> slot of its full-precision rows
   const int n_fp_old = L.n_fp;
-  const int64_t seen_old = L.n_seen, tile0 = L.n_quant / G;
+  const int64_t seen_old = L.n_seen;
   const std::vector<int32_t> old_tok(L.slot_token.begin(), L.slot_token.begin() + n_fp_old);
   std::vector<std::pair<int32_t, int32_t>> old_slots(n_fp_old);  // (token, slot), sorted by token
   for (int s = 0; s < n_fp_old; ++s) old_slots[s] = {old_tok[s], s};
@@ -754,12 +827,21 @@ lq_status_t ingest_prompt(lq_cache* c, int layer, const void* k, const void* v, 
     c->last_error = "ingestion plan failed its self-check";
     return LQ_ERR_CUDA;
   }
-  // pageable source: the runtime stages it before the call returns, so `idx` may die here
-  cudaError_t e = cudaMemcpyAsync(c->ingest_idx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) return cuda_fail(c, e, "prompt index upload");
-  e = launch_ingest(c->cv, layer, k, v, n, c->ingest_idx, n_tiles, has_fill, n_copy, tile0, c->sm_count, st);
-  if (e != cudaSuccess) return cuda_fail(c, e, "lq_ingest_kernel");
-  { c->n_launches++; c->last_decode_layer = -1; }
+  plan.n_tiles = n_tiles;
+  plan.n_copy = n_copy;
+  plan.has_fill = has_fill;
+  plan.idx_ints = static_cast<int64_t>(idx.size());
+  if (static_cast<int>(c->plans.size()) == kMaxIngestPlans || c->idx_used + plan.idx_ints > ingest_idx_ints(c)) {
+    c->plans.clear();
+    c->idx_used = 0;
+  }
+  plan.idx_at = c->idx_used;
+  copy_bookkeeping(plan.after, L);
+  plan.ids = std::move(ids);
+  const lq_status_t s = launch_plan(c, layer, plan, idx.data(), k, v, st);
+  if (s != LQ_OK) return s;
+  c->idx_used += (plan.idx_ints + 3) / 4 * 4;
+  c->plans.push_back(std::move(plan));
   return LQ_OK;
 }
 

@@ -66,6 +66,17 @@ cudaError_t launch_compress(const CacheView& cv, const LayerList& layers, const 
 cudaError_t launch_ingest(const CacheView& cv, int layer, const void* k, const void* v, int n_src, const int* idx_dev,
                           int n_tiles, bool has_fill, int n_copy, int64_t tile0, int sm_count, cudaStream_t st);
 
+// Guard bytes behind freshly allocated blocks, and zeros in the small ones that must start at rest: one launch.
+struct BlockInit {
+  int n_guards, n_zero;
+  uint8_t* guard[16];      // 256 bytes of kGuardPattern each
+  uint4* zero[4];
+  int64_t zero_chunks[4];  // 16-byte chunks
+};
+constexpr int kGuardBytes = 256;  // after every device block; checked by lq_check_guards
+constexpr int kGuardPattern = 0xA5;
+cudaError_t launch_init_blocks(const BlockInit& b, cudaStream_t st);
+
 // Canonical export of one layer into device buffers (any pointer may be null).
 // slot_of_rank[i] = fp slot of the i-th kept id (ascending ids); device array of n_fp ints.
 cudaError_t launch_export(const CacheView& cv, int layer, int n_fp, int64_t n_quant,

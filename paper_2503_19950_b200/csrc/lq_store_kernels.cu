@@ -662,6 +662,22 @@ cudaError_t launch_ingest(const CacheView& cv, int layer, const void* k, const v
 }
 
 // ---------------------------------------------------------------------------------------
+// Blocks of a new cache (launch latency: seventeen memset calls took 70 us of the host's time, this one 4).
+// ---------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) lq_init_blocks_kernel(BlockInit b) {
+  if (static_cast<int>(blockIdx.x) < b.n_guards) b.guard[blockIdx.x][threadIdx.x] = static_cast<uint8_t>(kGuardPattern);
+  for (int z = 0; z < b.n_zero; ++z)
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < b.zero_chunks[z]; i += gridDim.x * 256LL)
+      b.zero[z][i] = make_uint4(0u, 0u, 0u, 0u);
+}
+static_assert(kGuardBytes == 256, "one guard byte per thread");
+
+cudaError_t launch_init_blocks(const BlockInit& b, cudaStream_t st) {
+  lq_init_blocks_kernel<<<256, 256, 0, st>>>(b);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------------------
 // Canonical export (introspection; not on the hot path).
 // ---------------------------------------------------------------------------------------
 __global__ void lq_export_codes_kernel(CacheView cv, int layer, int64_t n_quant, uint8_t* k_codes,

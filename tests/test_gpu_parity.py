@@ -835,3 +835,29 @@ def test_fused_steps_of_many_layers_overlap_without_a_wait_per_step(L, expect_al
     cache.close()
     for oc in ocs:
         oc.close()
+
+
+@pytest.mark.parametrize("W,G,chunks", [(32, 32, [32 * 9 + 5]), (32, 32, [200, 70, 129]), (42, 64, [300, 200, 84, 85]),
+                                        (32, 32, [100] + [65] * 40)])
+def test_layers_that_share_an_ingestion_plan(W, G, chunks):
+    """Layers in the same state take the plan that the first one made (index lists on the device included); a layer in
+    another state, another stream and more chunks than plans are kept have it made again."""
+    B, Hq, Hkv, D, N = 2, 4, 2, 128, sum(chunks)
+    cache = LogQuantCache(4, B, Hq, Hkv, W, G, max_tokens=N + 8)
+    streams = [torch.cuda.current_stream(), torch.cuda.current_stream(), torch.cuda.Stream(), torch.cuda.current_stream()]
+    caches = []
+    for layer in range(4):
+        k, v = synth.keys_values(100 + layer, B, Hkv, N + 3, D, "cuda")
+        oc = oracle.OracleCache(B, Hq, Hkv, D, W, G)
+        at = 0
+        torch.cuda.synchronize()
+        for n in ([3] if layer == 3 else []) + chunks:   # the last layer is three tokens ahead of the others
+            with torch.cuda.stream(streams[layer]):
+                cache.append(layer, k[:, :, at:at + n].contiguous(), v[:, :, at:at + n].contiguous())
+            at += n
+        torch.cuda.synchronize()
+        oc.append(synth.bf16_bits(k[:, :, :at]), synth.bf16_bits(v[:, :, :at]))
+        caches.append(oc)
+    for layer, oc in enumerate(caches):
+        assert_images_equal(cache.export(layer), oc.export())
+    cache.close()
