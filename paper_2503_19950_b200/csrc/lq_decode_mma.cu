@@ -10,8 +10,11 @@
 // pair's partials and writes the output.
 //
 // Contractions (mma.sync.m16n8k16, fp32 accumulate), r = query heads per KV head (<= 8):
-//   q.k   tokens on M (16), query heads on N, channels on K.  Heads are handled in column blocks
-//         of 4: column 2h' = "hi", 2h'+1 = "lo" of head 4cb+h'.
+//   q.k   tokens on M (16), query heads on N, channels on K.
+//         r <= 4: column 2h = "hi", 2h+1 = "lo" of head h; r > 4: column h = head h, with one MMA for the hi parts
+//         and one for the lo parts on the same accumulators (against two blocks of four heads with hi and lo columns
+//         each: half the query fragments, score accumulators and q.zero products, GQA-7 at 32k 15.9 -> 14.5 us per
+//         layer, eight heads with 4-bit codes 31.3 -> 27.2 us).
 //         2-bit keys: the A fragment is the packed word masked at one code position -- a bf16
 //         subnormal c*2^(p-133) -- so unpacking costs one AND per two codes.  The key scale is
 //         folded into the query: q*s is split exactly into bf16 hi + lo with one packed multiply
@@ -52,6 +55,12 @@ constexpr int kWarpStageBytes = warp_stage_bytes(32);
 constexpr int kMaxStages = 3;
 constexpr int kOverlapDepth = 3;  // consecutive overlapped launches that share the SMs (plan_decode_mma)
 constexpr int kCtasPerSm = 4;  // at 128 registers and 51 KB of shared memory; 3 and 5 both measured slower
+// More than four query heads per KV head need 168 registers (at 128 they spill: 16.4 instead of 14.5 us per layer on the
+// GQA-7 workload); the 9 KB stages of 4-bit codes at G = 64 leave shared memory for three CTAs as well, and these then take
+// the registers too (21.4 -> 19.9 us, B = 8, 32/8 heads, 8192 tokens).
+__host__ __device__ constexpr int ctas_per_sm(int ncb, int G, int PL) {
+  return ncb == 2 || (G == 64 && PL == 2) ? kCtasPerSm - 1 : kCtasPerSm;
+}
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr int kSpinLimit = 1 << 22;
 // cost of one fp tile (16 bf16 tokens, two loads) in eighths of a quant tile: 4 to 12 measured alike,
@@ -198,7 +207,7 @@ template <int NCB>
 struct WarpState {
   float out[8][4];  // o^T: [channel tile][c-fragment]
   float zacc[4];    // sum_t p_t * vzero_t per (value group, column)
-  float m[NCB];     // running max (log2 units) of head 4cb + lane%4
+  float m[NCB];     // running max (log2 units) of head lane%4 (NCB == 1) or 2 (lane%4) + cb
   float l[NCB];     // this lane's share of the running denominator (times 2^kPExp)
   bool quant_mode;  // out rows carry the code-position factor
 };
@@ -214,11 +223,10 @@ __device__ __forceinline__ int vpos_log2(int mt) {
 }
 
 // ---- online softmax over the NSUB*16 scores of one tile ---------------------------------------
-// s[u][cb][th]: score (log2 units) of token 16u + 8th + lane/4 for head 4cb + lane%4; replaced by
+// s[u][cb][th]: score (log2 units) of token 16u + 8th + lane/4 for head lane%4 (NCB == 1) or 2 (lane%4) + cb; replaced by
 // the probabilities 2^(s - m + kPExp).
 template <int NCB, int NSUB>
 __device__ __forceinline__ void tile_softmax(WarpState<NCB>& st, float (&s)[NSUB][NCB][2], int lane, int opaque_zero) {
-  const int j = lane & 3;
   float corr[NCB];
   bool changed = false;
 #pragma unroll
@@ -242,14 +250,8 @@ __device__ __forceinline__ void tile_softmax(WarpState<NCB>& st, float (&s)[NSUB
   int again = __any_sync(kFull, changed);
   while (again) {
     float ca, cbv;
-    if (bf16_pv<NCB>()) {
-      ca = cbv = corr[0];  // all four accumulators of a lane belong to head lane%4
-    } else {
-      const float a0 = __shfl_sync(kFull, corr[0], (2 * j) & 3), a1 = __shfl_sync(kFull, corr[NCB - 1], (2 * j) & 3);
-      const float b0 = __shfl_sync(kFull, corr[0], (2 * j + 1) & 3), b1 = __shfl_sync(kFull, corr[NCB - 1], (2 * j + 1) & 3);
-      ca = j >= 2 ? a1 : a0;
-      cbv = j >= 2 ? b1 : b0;
-    }
+    ca = corr[0];  // r <= 4: all four accumulators of a lane belong to head lane%4
+    cbv = corr[NCB - 1];
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) {
       st.out[mt][0] *= ca; st.out[mt][1] *= cbv; st.out[mt][2] *= ca; st.out[mt][3] *= cbv;
@@ -287,9 +289,9 @@ __device__ __forceinline__ void transpose_p(const float (&p)[NCB][2], float (&pT
       } else if (NCB == 1) {
         pT[th][i] = __shfl_sync(kFull, p[0][th], 4 * (2 * j + i) + (n & 3));  // column n -> head n (mod 4)
       } else {
-        const int src = 4 * (2 * j + i) + (n & 3);  // column n -> head n
+        const int src = 4 * (2 * j + i) + (n >> 1);  // column n -> head n
         const float v0 = __shfl_sync(kFull, p[0][th], src), v1 = __shfl_sync(kFull, p[NCB - 1][th], src);
-        pT[th][i] = (n >> 2) ? v1 : v0;
+        pT[th][i] = (n & 1) ? v1 : v0;
       }
     }
 }
@@ -310,12 +312,12 @@ __device__ __forceinline__ void split_p_bf16(const float (&pT)[2][2], bool odd, 
 // units: the K rows (scores, softmax; leaves the p.v B operands in b0/b1), then the V rows -------
 // pad16: bit i set = slot i of the tile is padding (left out); at least one valid slot is not
 template <int NCB>
-__device__ __forceinline__ void process_fp_keys(WarpState<NCB>& st, const uint32_t (&qs)[NCB][8][2], uint32_t krows,
+__device__ __forceinline__ void process_fp_keys(WarpState<NCB>& st, const uint32_t (&qs)[8][2], uint32_t krows,
                                                 int n_valid, const float (&kc)[4], int lane, uint32_t oddmask,
                                                 int opaque_zero, uint32_t (&b0)[2], uint32_t (&b1)[2],
                                                 uint32_t pad16 = 0u) {
   const int n = lane >> 2;
-  float acc[NCB][4][4];
+  float acc[4][4];
   {
     const int mi = lane >> 3, rr = lane & 7;
     const int token = rr + 8 * (mi & 1);
@@ -325,21 +327,18 @@ __device__ __forceinline__ void process_fp_keys(WarpState<NCB>& st, const uint32
       const int chunk = 2 * ks + (mi >> 1);
       uint32_t a0, a1, a2, a3;
       ldmatrix_x4(rowaddr + ((chunk ^ (token & 7)) << 4), a0, a1, a2, a3);
-#pragma unroll
-      for (int cb = 0; cb < NCB; ++cb) {
-        if (ks < 4) mma_bf16_z(acc[cb][ks & 3], a0, a1, a2, a3, qs[cb][ks][0], qs[cb][ks][1]);
-        else mma_bf16(acc[cb][ks & 3], a0, a1, a2, a3, qs[cb][ks][0], qs[cb][ks][1]);
-      }
+      if (ks < 4) mma_bf16_z(acc[ks & 3], a0, a1, a2, a3, qs[ks][0], qs[ks][1]);
+      else mma_bf16(acc[ks & 3], a0, a1, a2, a3, qs[ks][0], qs[ks][1]);
     }
   }
   float s[1][NCB][2];
 #pragma unroll
   for (int cb = 0; cb < NCB; ++cb) {
-    float s0 = acc[cb][0][0] * kc[0], s1 = acc[cb][0][2] * kc[0];
+    float s0 = acc[0][cb] * kc[0], s1 = acc[0][2 + cb] * kc[0];
 #pragma unroll
     for (int c = 1; c < 4; ++c) {
-      s0 = fmaf(acc[cb][c][0], kc[c], s0);
-      s1 = fmaf(acc[cb][c][2], kc[c], s1);
+      s0 = fmaf(acc[c][cb], kc[c], s0);
+      s1 = fmaf(acc[c][2 + cb], kc[c], s1);
     }
     s[0][cb][0] = n < n_valid && !((pad16 >> n) & 1u) ? s0 : -INFINITY;
     s[0][cb][1] = n + 8 < n_valid && !((pad16 >> (n + 8)) & 1u) ? s1 : -INFINITY;
@@ -377,32 +376,29 @@ __device__ __forceinline__ void process_fp_values(WarpState<NCB>& st, uint32_t v
   }
 }
 
-// ---- q.zero of the key groups of one stage: bias[t][cb] for head 4cb + lane%4 of tile t (log2 units).
+// ---- q.zero of the key groups of one stage: bias[t][cb] for head lane%4 (2 (lane%4) + cb) of tile t (log2 units).
 // One MMA per k-step serves two tiles: the A fragment's rows 0-7 repeat the zero row of tile 0 and
 // rows 8-15 that of tile 1 (ldmatrix with equal row addresses inside each 8x8 matrix); the four
 // accumulators collect the k-steps of equal code-position factor, which kc[] undoes.
 // zaddr: this lane's row address, k-step 0.
 template <int NCB>
-__device__ __forceinline__ void quant_bias(const uint32_t (&qs)[NCB][8][2], uint32_t zaddr, const float (&kc)[4],
+__device__ __forceinline__ void quant_bias(const uint32_t (&qs)[8][2], uint32_t zaddr, const float (&kc)[4],
                                            float (&bias)[2][NCB]) {
-  float accb[NCB][4][4];
+  float accb[4][4];
 #pragma unroll
   for (int ks = 0; ks < 8; ++ks) {
     uint32_t z0, z1, z2, z3;
     ldmatrix_x4(zaddr + 32 * ks, z0, z1, z2, z3);
-#pragma unroll
-    for (int cb = 0; cb < NCB; ++cb) {
-      if (ks < 4) mma_bf16_z(accb[cb][ks & 3], z0, z1, z2, z3, qs[cb][ks][0], qs[cb][ks][1]);
-      else mma_bf16(accb[cb][ks & 3], z0, z1, z2, z3, qs[cb][ks][0], qs[cb][ks][1]);
-    }
+    if (ks < 4) mma_bf16_z(accb[ks & 3], z0, z1, z2, z3, qs[ks][0], qs[ks][1]);
+    else mma_bf16(accb[ks & 3], z0, z1, z2, z3, qs[ks][0], qs[ks][1]);
   }
 #pragma unroll
   for (int cb = 0; cb < NCB; ++cb) {
-    float b0 = accb[cb][0][0] * kc[0], b1 = accb[cb][0][2] * kc[0];
+    float b0 = accb[0][cb] * kc[0], b1 = accb[0][2 + cb] * kc[0];
 #pragma unroll
     for (int c = 1; c < 4; ++c) {
-      b0 = fmaf(accb[cb][c][0], kc[c], b0);
-      b1 = fmaf(accb[cb][c][2], kc[c], b1);
+      b0 = fmaf(accb[c][cb], kc[c], b0);
+      b1 = fmaf(accb[c][2 + cb], kc[c], b1);
     }
     bias[0][cb] = b0;
     bias[1][cb] = b1;
@@ -426,17 +422,18 @@ __device__ __forceinline__ void patch_new_row(uint32_t half_tile_smem, uint8_t* 
 // plane is added, and in p.v it meets p * s_v * 4 (all exact).
 // pad0/pad1: bit i set = token i (pad0) or 32 + i (pad1) of the tile is padding (left out); not all of them are
 template <int G, int NCB, int PL>
-__device__ __forceinline__ void process_quant_tile(WarpState<NCB>& st, const uint32_t (&qs)[NCB][8][2], uint32_t tile,
+__device__ __forceinline__ void process_quant_tile(WarpState<NCB>& st, const uint32_t (&qs)[8][2], uint32_t tile,
                                                    const float (&bias)[NCB], float kq, int lane, uint32_t oddmask,
                                                    int opaque_zero, uint32_t pad0 = 0u, uint32_t pad1 = 0u) {
   constexpr int NS = G / 16, NG = kD / G, VS = vsz_subtile_bytes(G);
   const int n = lane >> 2, j = lane & 3;
   // ---- q.k on all G tokens.  Per pair of k-steps: the key scale of the lane's channels is folded
-  // into the query (even columns RN(q*s), odd columns the exact residual) and every sub-tile's
-  // score accumulator advances by one MMA per k-step; the group's q.zero comes in as `bias`.
+  // into the query (hi = RN(q*s) and lo = the exact residual: in even and odd columns for r <= 4, else in two
+  // operands) and every sub-tile's score accumulator advances by one (two) MMAs per k-step; the group's q.zero
+  // comes in as `bias`.
   float s[NS][NCB][2];
   {
-    float acc[NS][NCB][4];
+    float acc[NS][4];
 #pragma unroll
     for (int pl = PL - 1; pl >= 0; --pl) {
       uint32_t kw[NS][4], kws[NS][4];
@@ -452,9 +449,7 @@ __device__ __forceinline__ void process_quant_tile(WarpState<NCB>& st, const uin
 #pragma unroll
         for (int u = 0; u < NS; ++u)
 #pragma unroll
-          for (int cb = 0; cb < NCB; ++cb)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[u][cb][e] *= 4.0f;
+          for (int e = 0; e < 4; ++e) acc[u][e] *= 4.0f;
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -463,35 +458,35 @@ __device__ __forceinline__ void process_quant_tile(WarpState<NCB>& st, const uin
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk) {
           const int ks = 2 * i + kk;
-          uint32_t bq[NCB][2];
+          uint32_t bq[2], lo[2];
 #pragma unroll
-          for (int cb = 0; cb < NCB; ++cb) {
-#pragma unroll
-            for (int w = 0; w < 2; ++w) {
-              // even columns RN(q*s); odd columns the exact residual q*s - RN(q*s)
-              bq[cb][w] = bf16x2_mul(qs[cb][ks][w], s4[2 * kk + w]);
-              if (oddmask) bq[cb][w] = bf16x2_fma(qs[cb][ks][w], s4[2 * kk + w], bf16x2_neg(bq[cb][w]));
-            }
+          for (int w = 0; w < 2; ++w) {
+            bq[w] = bf16x2_mul(qs[ks][w], s4[2 * kk + w]);
+            if (NCB == 2) lo[w] = bf16x2_fma(qs[ks][w], s4[2 * kk + w], bf16x2_neg(bq[w]));
+            else if (oddmask) bq[w] = bf16x2_fma(qs[ks][w], s4[2 * kk + w], bf16x2_neg(bq[w]));
           }
 #pragma unroll
           for (int u = 0; u < NS; ++u) {
             const uint32_t a0 = ext_bf16_i(ks, kw[u][0], kws[u][0]), a1 = ext_bf16_i(ks, kw[u][1], kws[u][1]),
                            a2 = ext_bf16_i(ks, kw[u][2], kws[u][2]), a3 = ext_bf16_i(ks, kw[u][3], kws[u][3]);
-#pragma unroll
-            for (int cb = 0; cb < NCB; ++cb) {
-              if (ks == 0 && pl == PL - 1) mma_bf16_z(acc[u][cb], a0, a1, a2, a3, bq[cb][0], bq[cb][1]);
-              else mma_bf16(acc[u][cb], a0, a1, a2, a3, bq[cb][0], bq[cb][1]);
-            }
+            if (ks == 0 && pl == PL - 1) mma_bf16_z(acc[u], a0, a1, a2, a3, bq[0], bq[1]);
+            else mma_bf16(acc[u], a0, a1, a2, a3, bq[0], bq[1]);
+            if (NCB == 2) mma_bf16(acc[u], a0, a1, a2, a3, lo[0], lo[1]);
           }
         }
       }
     }
 #pragma unroll
-    for (int cb = 0; cb < NCB; ++cb) {
+    for (int u = 0; u < NS; ++u) {
+      if (NCB == 1) {
+        s[u][0][0] = fmaf(acc[u][0] + acc[u][1], kq, bias[0]);
+        s[u][0][1] = fmaf(acc[u][2] + acc[u][3], kq, bias[0]);
+      } else {
 #pragma unroll
-      for (int u = 0; u < NS; ++u) {
-        s[u][cb][0] = fmaf(acc[u][cb][0] + acc[u][cb][1], kq, bias[cb]);
-        s[u][cb][1] = fmaf(acc[u][cb][2] + acc[u][cb][3], kq, bias[cb]);
+        for (int cb = 0; cb < NCB; ++cb) {
+          s[u][cb][0] = fmaf(acc[u][cb], kq, bias[cb]);
+          s[u][cb][1] = fmaf(acc[u][2 + cb], kq, bias[cb]);
+        }
       }
     }
     if (pad0 | pad1) {  // always false in the instantiation without padding (constant arguments)
@@ -634,7 +629,7 @@ constexpr int kMergeOneBatch = 12;  // CTA records the fused second pass loads i
 // PADDED: the batch is left-padded (DecodeArgs::rowinfo): per sequence, leading quant tiles that are
 // padding entirely are not visited, and tiles and slots with padding among their tokens get -inf scores.
 template <int G, int NCB, int PL, bool FUSED, bool PADDED>
-__global__ void __launch_bounds__(kWarps * 32, NCB == 1 ? kCtasPerSm : kCtasPerSm - 1) lq_decode_mma_kernel(DecodeArgs a) {
+__global__ void __launch_bounds__(kWarps * 32, ctas_per_sm(NCB, G, PL)) lq_decode_mma_kernel(DecodeArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   const CacheView& cv = a.cv;
   const int r = cv.Hq / cv.Hkv;
@@ -786,9 +781,9 @@ __global__ void __launch_bounds__(kWarps * 32, NCB == 1 ? kCtasPerSm : kCtasPerS
     issue_next(1);
   }
 
-  // query fragments: B operand, column n -> head 4cb + n/2 (even column = hi, odd = lo of q*s);
+  // query fragments: B operand, column n -> head n/2 (even column = hi, odd = lo of q*s), for r > 4 head n;
   // k-step ks carries the factor 2^(64 - 2*(ks&3)) that cancels the code-position factor
-  uint32_t qs[NCB][8][2];
+  uint32_t qs[8][2];
   // Pairs with more CTAs than the last one could fetch the records of in one batch of loads (kMergeOneBatch):
   // every CTA also adds its partial to one sum per pair (DecodeArgs::acc), scaled to a reference score that
   // all of them compute alike: q . k of the token in fp slot 0 (any real score of the pair will do).  Thread
@@ -815,9 +810,8 @@ __global__ void __launch_bounds__(kWarps * 32, NCB == 1 ? kCtasPerSm : kCtasPerS
         if (lane == h) ref = dot * a.scale_log2;
       }
     }
-#pragma unroll
-    for (int cb = 0; cb < NCB; ++cb) {
-      const int head = 4 * cb + (n >> 1);
+    {
+      const int head = NCB == 1 ? n >> 1 : n;
       const bool valid = head < r;
       const uint32_t qrow = qsm + (valid ? head : 0) * (kD * 2);
 #pragma unroll
@@ -828,7 +822,7 @@ __global__ void __launch_bounds__(kWarps * 32, NCB == 1 ? kCtasPerSm : kCtasPerS
           asm volatile("ld.shared.u32 %0, [%1];" : "=r"(raw) : "r"(qrow + 2 * (16 * ks + 8 * w + 2 * j)));
           // 2^(64 - 2*(ks&3)) as a bf16 pair: the product is exact (a power of two, no overflow)
           const uint32_t f2 = (static_cast<uint32_t>(127 + 64 - 2 * (ks & 3)) << 7) * 0x00010001u;
-          qs[cb][ks][w] = valid ? bf16x2_mul(raw, f2) : 0u;
+          qs[ks][w] = valid ? bf16x2_mul(raw, f2) : 0u;
         }
     }
   }
@@ -984,8 +978,8 @@ __global__ void __launch_bounds__(kWarps * 32, NCB == 1 ? kCtasPerSm : kCtasPerS
   if (n == 0) {
 #pragma unroll
     for (int cb = 0; cb < NCB; ++cb) {
-      wm[warp * 8 + 4 * cb + j] = st.m[cb];
-      wl[warp * 8 + 4 * cb + j] = st.l[cb];
+      wm[warp * 8 + NCB * j + cb] = st.m[cb];
+      wl[warp * 8 + NCB * j + cb] = st.l[cb];
     }
   }
   __syncthreads();
@@ -1244,12 +1238,12 @@ void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_overrid
   // at most one resident wave of CTAs in total: a CTA that had to wait for a free slot would start
   // when the others finish, and its pair's merge would wait for it
   // the two-column-block variant needs more registers, the 9 KB stages of 4-bit codes at G = 64 more shared memory
-  const int ctas_per_sm = r <= 4 && !(a.cv.G == 64 && a.cv.planes == 2) ? kCtasPerSm : kCtasPerSm - 1;
+  const int n_ctas_sm = ctas_per_sm(r <= 4 ? 1 : 2, a.cv.G, a.cv.planes);
   // A serialised launch fills exactly one resident wave.  An overlapped launch (DecodeArgs::early) takes a third of
   // the slots with CTAs three times as long (at least one CTA per pair): three consecutive launches then share the
   // SMs, every slot stays busy, and the fixed costs of a CTA (start-up, merge, ticket: 4 - 5 us) are paid once per
   // three times the bytes (measured: 1/2 and 1/3 alike, 1/4 worse; 8k workload 15.4 -> 14.4 us per launch).
-  const int wave = a.early ? std::max(pairs, ctas_per_sm * sm_count / kOverlapDepth) : ctas_per_sm * sm_count;
+  const int wave = a.early ? std::max(pairs, n_ctas_sm * sm_count / kOverlapDepth) : n_ctas_sm * sm_count;
   int S = s_override > 0 ? s_override : wave / pairs;
   S = std::min(S, (items + kWarps - 1) / kWarps);  // at least one item per warp
   S = std::min(S, max_records - 1);
@@ -1277,7 +1271,7 @@ int plan_decode_mma_padded(const DecodeArgs& a, int sm_count, int max_records, c
   const int tiles_fp = (a.n_fp + kFpTileSlots - 1) / kFpTileSlots;
   const int tiles_quant = static_cast<int>(a.n_quant / a.cv.G);
   const int tps = stage_bytes(a.cv.G, a.cv.planes) / quant_tile_bytes(a.cv.G, a.cv.planes);
-  const int slots = (r <= 4 && !(a.cv.G == 64 && a.cv.planes == 2) ? kCtasPerSm : kCtasPerSm - 1) * sm_count;
+  const int slots = ctas_per_sm(r <= 4 ? 1 : 2, a.cv.G, a.cv.planes) * sm_count;
   const int wave = overlapped ? std::max(pairs, slots / kOverlapDepth) : slots;  // as in plan_decode_mma
   const int cap_records = std::max(1, std::min(max_records, kMergeMax / r));
   std::vector<int64_t> work(pairs);
