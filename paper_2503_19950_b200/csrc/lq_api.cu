@@ -74,6 +74,7 @@ struct lq_cache {
   // LQ_FLAG_OVERLAP_DECODE: layer and stream of the decode launch that was this cache's last enqueued work (-1: the
   // last work was something else)
   int last_decode_layer = -1;
+  int last_row_layer = -1;  // layer to which that launch appended a row (-1: none)
   cudaStream_t last_decode_stream = nullptr;
   // Rows written by fused append+attention launches that may still be running.  An overlapped launch of the same
   // layer reads that row in its main loop, before its dependency wait, so it may overlap only when the writing
@@ -1061,6 +1062,7 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
   a.zero = 0;
   a.n_extra = 0;
   a.early = 0;
+  a.small = a.prefetch = 0;
   if (use_mma(c)) {
     if (c->row_mark.empty()) c->row_mark.assign(c->cfg.n_layers, -1);
     // twice the CTAs of these kernels the device can hold (51 KB of shared memory each: at most four per SM)
@@ -1083,6 +1085,12 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
       a.n_extra = 0;
     }
     c->ctas_since_wait += a.rowinfo ? a.n_ctas : c->cfg.batch * c->cfg.n_kv_heads * (a.S - 1) + a.n_extra;  // the grid
+    // A small launch may read its stores before it waits for the launch before it, if that was this cache's last work, a
+    // decode launch on the same stream (so that everything older has finished: it waited at entry itself) and did not write
+    // a row of this layer.
+    if (a.rowinfo || (c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) || timed) a.small = 0;
+    a.prefetch = a.small && c->last_decode_layer >= 0 && c->last_row_layer != layer && c->last_decode_stream == st;
+    c->last_row_layer = new_k != nullptr ? layer : -1;
     if (a.early) c->n_overlapped++;
     c->row_mark[layer] = new_k != nullptr ? c->ctas_since_wait : -1;
     a.tickets = c->tickets;  // the CTA that completes a (b, kv) pair merges it: no second launch

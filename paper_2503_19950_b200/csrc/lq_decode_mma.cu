@@ -705,28 +705,6 @@ __global__ void __launch_bounds__(kWarps * 32, ctas_per_sm(NCB, G, PL)) lq_decod
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
-  // Programmatic dependent launch: everything above touches only this CTA's shared memory, the launch
-  // arguments and, in the padded variant, the CTA map and row info of the mask block -- which only a host copy
-  // enqueued by the same call writes (upload_masks), never a kernel that could still be running.  Nothing an
-  // earlier kernel may still be writing is read before it has finished.
-  if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
-  // In a chain of overlapped launches the next launch may take the slots of this one as soon as they free up (its
-  // CTAs stream their own layer and wait for this grid only before the workspace); otherwise the trigger comes
-  // after the main loop, so that CTAs that could only wait do not take the slots earlier.
-  if (a.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (threadIdx.x == 0) {
-    // the r query rows of this pair are contiguous: one bulk copy
-    mbar_expect_tx(qbar, r * kD * 2);
-    if (!a.debug_stall)
-      bulk_load(qsm, static_cast<const uint8_t*>(a.q) + (static_cast<int64_t>(b) * cv.Hq + kv * r) * kD * 2, r * kD * 2,
-                qbar);
-  }
-
-  float kc[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) kc[c] = a.scale_log2 * pow2i(2 * c - 64);
-  const float kq = a.scale_log2 * pow2i(69);
-
   const uint8_t* fpbase = cv.fp + a.layer * cv.fp_layer_stride + pair * cv.fp_head_stride;
   const uint8_t* qbase = cv.quant + a.layer * cv.quant_layer_stride + pair * cv.quant_head_stride;
 
@@ -771,15 +749,42 @@ __global__ void __launch_bounds__(kWarps * 32, ctas_per_sm(NCB, G, PL)) lq_decod
     }
     ++issued;
   };
+  // A small launch whose predecessor on the stream did not write this layer (DecodeArgs::prefetch) fetches its stages now,
+  // while that launch still merges.
+  if (a.prefetch) {
+#pragma unroll 1
+    for (int s = 0; s < kStages; ++s) issue_next(TPS);
+  }
+  // Programmatic dependent launch: everything above touches only this CTA's shared memory, the launch
+  // arguments and, in the padded variant, the CTA map and row info of the mask block -- which only a host copy
+  // enqueued by the same call writes (upload_masks), never a kernel that could still be running.  Nothing an
+  // earlier kernel may still be writing is read before it has finished.
+  if (!a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // In a chain of overlapped launches the next launch may take the slots of this one as soon as they free up (its
+  // CTAs stream their own layer and wait for this grid only before the workspace); otherwise the trigger comes
+  // after the main loop, so that CTAs that could only wait do not take the slots earlier.
+  // (small launches likewise, once everything before them has finished: the next one may then fetch its stages)
+  if (a.early || a.small) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (threadIdx.x == 0) {
+    // the r query rows of this pair are contiguous: one bulk copy
+    mbar_expect_tx(qbar, r * kD * 2);
+    if (!a.debug_stall)
+      bulk_load(qsm, static_cast<const uint8_t*>(a.q) + (static_cast<int64_t>(b) * cv.Hq + kv * r) * kD * 2, r * kD * 2,
+                qbar);
+  }
+
+  float kc[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) kc[c] = a.scale_log2 * pow2i(2 * c - 64);
+  const float kq = a.scale_log2 * pow2i(69);
+
   bool failed = false;
   // Only one small load per warp before the query fragments are built: all warps start at the same
   // time, and the first bytes every warp needs should not queue behind everybody's second load.
   // (an overlapped launch starts while other CTAs of the SM are in mid-stream: it fills all its stages at once)
-  if (a.early) {
-    for (int s = 0; s < kStages; ++s) issue_next(TPS);
-  } else {
-    issue_next(1);
-  }
+#pragma unroll 1
+  for (int s = issued; s < (a.early ? kStages : 1); ++s) issue_next(a.early ? TPS : 1);
+
 
   // query fragments: B operand, column n -> head n/2 (even column = hi, odd = lo of q*s), for r > 4 head n;
   // k-step ks carries the factor 2^(64 - 2*(ks&3)) that cancels the code-position factor
@@ -826,8 +831,10 @@ __global__ void __launch_bounds__(kWarps * 32, ctas_per_sm(NCB, G, PL)) lq_decod
         }
     }
   }
-  if (!a.early)
-    for (int s = 1; s < kStages; ++s) issue_next(TPS);
+  if (!a.early) {
+#pragma unroll 1
+    for (int s = issued; s < kStages; ++s) issue_next(TPS);
+  }
   WarpState<NCB> st;
 #pragma unroll
   for (int mt = 0; mt < 8; ++mt) st.out[mt][0] = st.out[mt][1] = st.out[mt][2] = st.out[mt][3] = 0.f;
@@ -911,7 +918,7 @@ __global__ void __launch_bounds__(kWarps * 32, ctas_per_sm(NCB, G, PL)) lq_decod
   }
   // the main loop is over: from here on the next kernel of the stream may start launching into
   // the slots that free up (earlier, its waiting CTAs would only take issue slots from this loop)
-  if (!a.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!a.early && !a.small) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // an overlapped launch (DecodeArgs::early) has read only its own layer's stores so far; the workspace below is
   // shared with the launch before it
   if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1246,6 +1253,12 @@ void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_overrid
   const int wave = a.early ? std::max(pairs, n_ctas_sm * sm_count / kOverlapDepth) : n_ctas_sm * sm_count;
   int S = s_override > 0 ? s_override : wave / pairs;
   S = std::min(S, (items + kWarps - 1) / kWarps);  // at least one item per warp
+  // A serialised launch that leaves half of the slots empty is nothing but latency.  Its warps then take single tiles, up to
+  // that half (one layer of 2 KV heads, 1024 tokens: 6.6 -> 5.8 us; beyond the half it costs, 8.2 -> 9.0 us for 8 KV heads,
+  // 8192 tokens), and the next launch may move into the other half and fetch its stages (DecodeArgs::prefetch: 8.9 -> 8.2 us
+  // there; without free slots it costs, 13.4 -> 15.4 us at 32768 tokens).
+  a.small = !a.early && s_override <= 0 && 2 * S * pairs <= wave;
+  if (a.small) S = std::max(S, std::min((a.tiles_fp + a.tiles_quant + kWarps - 1) / kWarps, wave / 2 / pairs));
   S = std::min(S, max_records - 1);
   S = std::min(S, kMergeMax / r - 1);
   S = std::max(S, 1);

@@ -150,6 +150,9 @@ struct DecodeArgs {
   // of the same cache (LQ_FLAG_OVERLAP_DECODE): nothing the main loop reads is written by it, so the dependency
   // wait of the programmatic launch moves behind the main loop, in front of the first use of the shared workspace
   int early;
+  // tensor-core kernel: a launch that leaves at least half of the SMs' slots free (plan_decode_mma); with prefetch, nothing
+  // its main loop reads from the stores is written by the launch before it on the stream
+  int small, prefetch;
 };
 
 constexpr int kAccStride = kMaxRatio * 128 + 32;  // floats per (b, kv) pair in DecodeArgs::acc

@@ -861,3 +861,45 @@ def test_layers_that_share_an_ingestion_plan(W, G, chunks):
     for layer, oc in enumerate(caches):
         assert_images_equal(cache.export(layer), oc.export())
     cache.close()
+
+
+@pytest.mark.parametrize("L,B,Hq,Hkv,n_prefill,two_streams", [(1, 1, 8, 2, 95, False), (2, 1, 8, 2, 200, False), (3, 2, 14, 2, 93, False),
+                                                              (3, 1, 4, 4, 33, True), (2, 3, 16, 8, 150, True)])
+def test_small_serialised_launches_that_fetch_their_stages_early(L, B, Hq, Hkv, n_prefill, two_streams):
+    """Default flags, few CTAs: a launch reads the stores of its layer before it waits for the launch before it.  Fused
+    steps across overflows, a plain repeat of the same layer right behind a fused step, layers in turn and streams in turn."""
+    W, G, D, steps = 32, 32, 128, 40
+    cache = LogQuantCache(L, B, Hq, Hkv, W, G, max_tokens=n_prefill + steps + 4)
+    oracles, data = [], []
+    for layer in range(L):
+        k, v = synth.keys_values(300 + layer, B, Hkv, n_prefill + steps, D, "cuda")
+        cache.append(layer, k[:, :, :n_prefill].contiguous(), v[:, :, :n_prefill].contiguous())
+        oracles.append(oracle.OracleCache(B, Hq, Hkv, D, W, G))
+        oracles[-1].append(synth.bf16_bits(k[:, :, :n_prefill]), synth.bf16_bits(v[:, :, :n_prefill]))
+        data.append((k, v))
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()] if two_streams else [torch.cuda.current_stream()] * 2
+    out = torch.empty(steps, L, 2, B, Hq, D, device="cuda")
+    qs = [[synth.queries(40 + layer, B, Hq, D, s, "cuda") for layer in range(L)] for s in range(steps)]
+    rows = [[tuple(x[:, :, n_prefill + s:n_prefill + s + 1].contiguous() for x in data[layer]) for layer in range(L)]
+            for s in range(steps)]
+    torch.cuda.synchronize()
+    for s in range(steps):
+        here = streams[s % 2]
+        here.wait_stream(streams[1 - s % 2])
+        with torch.cuda.stream(here):
+            for layer in range(L):
+                cache.append_decode_attn(layer, *rows[s][layer], qs[s][layer], out[s, layer, 0])
+                if s % 3 == 0:
+                    cache.decode_attn(layer, qs[s][layer], out[s, layer, 1])
+    torch.cuda.synchronize()
+    got = out.cpu().numpy()
+    for s in range(steps):
+        for layer in range(L):
+            oracles[layer].append(*(synth.bf16_bits(x) for x in rows[s][layer]))
+            ref = oracles[layer].attention(synth.bf16_bits(qs[s][layer]), 1 / np.sqrt(D), n_threads=8)
+            for i in range(2 if s % 3 == 0 else 1):
+                assert np.abs(got[s, layer, i] - ref).max() <= attn_tolerance(ref), (s, layer, i)
+    for layer in range(L):
+        assert_images_equal(cache.export(layer), oracles[layer].export())
+    assert cache.kernel_status() == 0
+    cache.close()
