@@ -417,9 +417,13 @@ __device__ __forceinline__ void patch_new_row(uint32_t half_tile_smem, uint8_t* 
 }
 
 // ---- one quant tile: one key group of G tokens ---------------------------------------------
-// PL = 2-bit planes per code.  A 4-bit code is 4 * (high plane) + (low plane): the high plane goes
-// through the same contractions first, its score accumulators are multiplied by 4 before the low
-// plane is added, and in p.v it meets p * s_v * 4 (all exact).
+// PL = 2-bit planes per code.  A 4-bit code is 4 * (high plane) + (low plane).  In q.k, up to 4 heads and G = 32, the low
+// plane meets a quarter of q * s and the sum counts four times: the key scale is folded in once for both planes
+// (22.2 -> 21.6 us per layer, B = 8, 32/8 heads, 8192 tokens).  With more heads, where q * s takes two operands, and at
+// G = 64 that costs registers (27.2 -> 28.7 us, 64/8 heads; 19.9 -> 20.0 us): the high plane goes first and its accumulators
+// are multiplied by 4 before the low plane is added.  In p.v the high plane meets p * s_v * 4 (all exact).
+template <int G, int NCB, int PL>
+__host__ __device__ constexpr int planes_together() { return G == 32 && NCB == 1 ? PL : 1; }
 // pad0/pad1: bit i set = token i (pad0) or 32 + i (pad1) of the tile is padding (left out); not all of them are
 template <int G, int NCB, int PL>
 __device__ __forceinline__ void process_quant_tile(WarpState<NCB>& st, const uint32_t (&qs)[8][2], uint32_t tile,
@@ -434,18 +438,21 @@ __device__ __forceinline__ void process_quant_tile(WarpState<NCB>& st, const uin
   float s[NS][NCB][2];
   {
     float acc[NS][4];
+    constexpr int kTogether = planes_together<G, NCB, PL>(), kPasses = PL / kTogether;
 #pragma unroll
-    for (int pl = PL - 1; pl >= 0; --pl) {
-      uint32_t kw[NS][4], kws[NS][4];
+    for (int pass = kPasses - 1; pass >= 0; --pass) {
+      uint32_t kw[kTogether][NS][4], kws[kTogether][NS][4];
 #pragma unroll
-      for (int u = 0; u < NS; ++u) {
-        const uint4 w = lds128(tile + qt_kcodes_off() + pl * qt_plane_bytes(G) + u * 512 + 16 * lane);
-        // words: (nt0,w0) (nt0,w1) (nt1,w0) (nt1,w1);  a0=(nt0,w0) a1=(nt1,w0) a2=(nt0,w1) a3=(nt1,w1)
-        kw[u][0] = w.x; kw[u][1] = w.z; kw[u][2] = w.y; kw[u][3] = w.w;
+      for (int pl = 0; pl < kTogether; ++pl)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) kws[u][e] = kw[u][e] >> 8;
-      }
-      if (pl != PL - 1) {
+        for (int u = 0; u < NS; ++u) {
+          const uint4 w = lds128(tile + qt_kcodes_off() + (pass + pl) * qt_plane_bytes(G) + u * 512 + 16 * lane);
+          // words: (nt0,w0) (nt0,w1) (nt1,w0) (nt1,w1);  a0=(nt0,w0) a1=(nt1,w0) a2=(nt0,w1) a3=(nt1,w1)
+          kw[pl][u][0] = w.x; kw[pl][u][1] = w.z; kw[pl][u][2] = w.y; kw[pl][u][3] = w.w;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) kws[pl][u][e] = kw[pl][u][e] >> 8;
+        }
+      if (pass != kPasses - 1) {
 #pragma unroll
         for (int u = 0; u < NS; ++u)
 #pragma unroll
@@ -466,12 +473,19 @@ __device__ __forceinline__ void process_quant_tile(WarpState<NCB>& st, const uin
             else if (oddmask) bq[w] = bf16x2_fma(qs[ks][w], s4[2 * kk + w], bf16x2_neg(bq[w]));
           }
 #pragma unroll
-          for (int u = 0; u < NS; ++u) {
-            const uint32_t a0 = ext_bf16_i(ks, kw[u][0], kws[u][0]), a1 = ext_bf16_i(ks, kw[u][1], kws[u][1]),
-                           a2 = ext_bf16_i(ks, kw[u][2], kws[u][2]), a3 = ext_bf16_i(ks, kw[u][3], kws[u][3]);
-            if (ks == 0 && pl == PL - 1) mma_bf16_z(acc[u], a0, a1, a2, a3, bq[0], bq[1]);
-            else mma_bf16(acc[u], a0, a1, a2, a3, bq[0], bq[1]);
-            if (NCB == 2) mma_bf16(acc[u], a0, a1, a2, a3, lo[0], lo[1]);
+          for (int pl = kTogether - 1; pl >= 0; --pl) {
+            if (pl != kTogether - 1) {  // the low plane counts a quarter
+#pragma unroll
+              for (int w = 0; w < 2; ++w) bq[w] = bf16x2_mul(bq[w], 0x3E803E80u);
+            }
+#pragma unroll
+            for (int u = 0; u < NS; ++u) {
+              const uint32_t a0 = ext_bf16_i(ks, kw[pl][u][0], kws[pl][u][0]), a1 = ext_bf16_i(ks, kw[pl][u][1], kws[pl][u][1]),
+                             a2 = ext_bf16_i(ks, kw[pl][u][2], kws[pl][u][2]), a3 = ext_bf16_i(ks, kw[pl][u][3], kws[pl][u][3]);
+              if (ks == 0 && pass == kPasses - 1 && pl == kTogether - 1) mma_bf16_z(acc[u], a0, a1, a2, a3, bq[0], bq[1]);
+              else mma_bf16(acc[u], a0, a1, a2, a3, bq[0], bq[1]);
+              if (NCB == 2) mma_bf16(acc[u], a0, a1, a2, a3, lo[0], lo[1]);
+            }
           }
         }
       }
@@ -776,7 +790,7 @@ __global__ void __launch_bounds__(kWarps * 32, ctas_per_sm(NCB, G, PL)) lq_decod
   float kc[4];
 #pragma unroll
   for (int c = 0; c < 4; ++c) kc[c] = a.scale_log2 * pow2i(2 * c - 64);
-  const float kq = a.scale_log2 * pow2i(69);
+  const float kq = a.scale_log2 * pow2i(planes_together<G, NCB, PL>() == 2 ? 71 : 69);
 
   bool failed = false;
   // Only one small load per warp before the query fragments are built: all warps start at the same
