@@ -1264,7 +1264,13 @@ void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_overrid
   // the slots with CTAs three times as long (at least one CTA per pair): three consecutive launches then share the
   // SMs, every slot stays busy, and the fixed costs of a CTA (start-up, merge, ticket: 4 - 5 us) are paid once per
   // three times the bytes (measured: 1/2 and 1/3 alike, 1/4 worse; 8k workload 15.4 -> 14.4 us per launch).
-  const int wave = a.early ? std::max(pairs, n_ctas_sm * sm_count / kOverlapDepth) : n_ctas_sm * sm_count;
+  // Above 256 MB per launch half of the slots do as well: the fixed costs no longer count, and the last launch of a series, which
+  // has nobody to share the SMs with, is over sooner (32 KV heads at 131072 tokens, four layers in a row and nothing behind them:
+  // 553 -> 484 us, among other passes 411 us either way; 47 to 116 MB per launch lose 1 to 7 %).
+  const int64_t bytes = static_cast<int64_t>(pairs) * (static_cast<int64_t>(a.tiles_fp) * kFpTileBytes +
+                                                       static_cast<int64_t>(a.tiles_quant) * quant_tile_bytes(a.cv.G, a.cv.planes));
+  const int depth = bytes > (256LL << 20) ? 2 : kOverlapDepth;
+  const int wave = a.early ? std::max(pairs, n_ctas_sm * sm_count / depth) : n_ctas_sm * sm_count;
   int S = s_override > 0 ? s_override : wave / pairs;
   S = std::min(S, (items + kWarps - 1) / kWarps);  // at least one item per warp
   // A serialised launch that leaves half of the slots empty is nothing but latency.  Its warps then take single tiles, up to
