@@ -277,6 +277,10 @@ lq_status_t lq_debug_stall_next_decode(lq_cache_t* cache);
  * written): destroy it. */
 lq_status_t lq_debug_bad_slot_next_append(lq_cache_t* cache);
 
+/* Test hook: number of decode-attention launches of this cache so far (all layers) that fetched their first tiles before
+ * they waited for the launch before them (see LQ_FLAG_OVERLAP_DECODE; host-side bookkeeping, never synchronises). */
+lq_status_t lq_debug_launches_prefetched(const lq_cache_t* cache, int64_t* n_launches);
+
 /* Guard words: every device block a cache allocates (through cudaMalloc or the caller's allocator) is
  * followed by 256 guard bytes of a fixed pattern that no kernel may touch.  lq_check_guards synchronises the
  * device, reads them back and stores the number of blocks whose guard was overwritten in *n_damaged

@@ -54,7 +54,8 @@ SYMBOLS = ["lq_cache_create", "lq_destroy", "lq_append", "lq_compress", "lq_deco
            "lq_decode_attn_fp_only", "lq_set_padding",
            "lq_decode_step_host", "lq_profile_enable", "lq_profile_read", "lq_kernel_status", "lq_cache_info", "lq_export",
            "lq_next_evicted_ids", "lq_decode_attn_image_static", "lq_status_str", "lq_last_error", "lq_check_guards",
-           "lq_reset_kernel_status", "lq_debug_stall_next_decode", "lq_debug_bad_slot_next_append", "lq_import"]
+           "lq_reset_kernel_status", "lq_debug_stall_next_decode", "lq_debug_bad_slot_next_append", "lq_import",
+           "lq_debug_launches_prefetched"]
 
 _lib = None
 
@@ -88,6 +89,7 @@ def load_library():
         L.lq_reset_kernel_status.argtypes = [vp]
         L.lq_debug_stall_next_decode.argtypes = [vp]
         L.lq_debug_bad_slot_next_append.argtypes = [vp]
+        L.lq_debug_launches_prefetched.argtypes = [vp, C.POINTER(C.c_int64)]
         L.lq_profile_enable.argtypes = [vp, i32]
         L.lq_profile_read.argtypes = [vp, C.POINTER(C.c_double), C.POINTER(C.c_int64)]
         L.lq_cache_info.argtypes = [vp, i32, C.POINTER(lq_info_t)]
@@ -293,6 +295,11 @@ class LogQuantCache:
 
     def debug_stall_next_decode(self):
         self._check(self._lib.lq_debug_stall_next_decode(self._h))
+
+    def debug_launches_prefetched(self) -> int:
+        n = C.c_int64(0)
+        self._check(self._lib.lq_debug_launches_prefetched(self._h, C.byref(n)))
+        return n.value
 
     def kernel_status(self) -> int:
         w = C.c_int32(0)

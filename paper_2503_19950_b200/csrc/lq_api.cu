@@ -88,6 +88,7 @@ struct lq_cache {
   std::vector<int64_t> row_mark;
   int64_t ctas_since_wait = 0;
   int32_t n_overlapped = 0;  // launches that took the overlapped form (lq_info_t::n_launches_overlapped)
+  int64_t n_prefetched = 0;  // launches that fetched their stages before the dependency wait (lq_debug_launches_prefetched)
   bool bad_slot_next = false;  // lq_debug_bad_slot_next_append (index-check build only)
   // left padding of a ragged batch (lq_set_padding): pad[b] leading positions of sequence b that attention
   // leaves out.  Device copy per layer: [B][4] row info, [B][fp_words] slot mask, [B][q_words] store mask,
@@ -115,6 +116,7 @@ lq_status_t cuda_fail(lq_cache* c, cudaError_t e, const char* what) {
   char buf[256];
   std::snprintf(buf, sizeof buf, "%s: %s", what, cudaGetErrorString(e));
   if (c) c->last_error = buf;
+  cudaGetLastError();  // (else the next launch that asks for its error would be told of this one)
   return LQ_ERR_CUDA;
 }
 
@@ -1070,10 +1072,6 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
     const bool row_safe = c->row_mark[layer] < 0 || c->ctas_since_wait - c->row_mark[layer] >= resident_bound;
     a.early = (c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) && !timed && c->last_decode_layer >= 0 &&
               c->last_decode_layer != layer && c->last_decode_stream == st && row_safe;
-    if (!a.early) {
-      std::fill(c->row_mark.begin(), c->row_mark.end(), -1);
-      c->ctas_since_wait = 0;
-    }
     plan_decode_mma(a, c->sm_count, c->max_splits, c->cfg.n_splits);
     if (a.rowinfo) {
       a.S = a.early ? c->pad_stride_ov[layer] : c->pad_stride[layer];
@@ -1084,19 +1082,26 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
       }
       a.n_extra = 0;
     }
-    c->ctas_since_wait += a.rowinfo ? a.n_ctas : c->cfg.batch * c->cfg.n_kv_heads * (a.S - 1) + a.n_extra;  // the grid
     // A small launch may read its stores before it waits for the launch before it, if that was this cache's last work, a
     // decode launch on the same stream (so that everything older has finished: it waited at entry itself) and did not write
     // a row of this layer.
     if (a.rowinfo || (c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) || timed) a.small = 0;
     a.prefetch = a.small && c->last_decode_layer >= 0 && c->last_row_layer != layer && c->last_decode_stream == st;
-    c->last_row_layer = new_k != nullptr ? layer : -1;
-    if (a.early) c->n_overlapped++;
-    c->row_mark[layer] = new_k != nullptr ? c->ctas_since_wait : -1;
     a.tickets = c->tickets;  // the CTA that completes a (b, kv) pair merges it: no second launch
     a.acc = c->acc;
+    // (a launch that fails is none: the next one derives nothing from it, nor from the one before it)
+    c->last_decode_layer = -1;
     e = launch_decode_mma(a, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "lq_decode_mma_kernel");
+    if (!a.early) {
+      std::fill(c->row_mark.begin(), c->row_mark.end(), -1);
+      c->ctas_since_wait = 0;
+    }
+    c->ctas_since_wait += a.rowinfo ? a.n_ctas : c->cfg.batch * c->cfg.n_kv_heads * (a.S - 1) + a.n_extra;  // the grid
+    c->row_mark[layer] = new_k != nullptr ? c->ctas_since_wait : -1;
+    c->last_row_layer = new_k != nullptr ? layer : -1;
+    if (a.early) c->n_overlapped++;
+    if (a.prefetch) c->n_prefetched++;
   } else if (use_umma(c)) {
     plan_decode_umma(a, c->sm_count, c->max_splits, c->cfg.n_splits);
     a.tickets = c->tickets;
@@ -1244,6 +1249,12 @@ lq_status_t lq_debug_bad_slot_next_append(lq_cache_t* c) {
 lq_status_t lq_debug_stall_next_decode(lq_cache_t* c) {
   if (!c) return LQ_ERR_INVALID_ARG;
   c->stall_next = true;
+  return LQ_OK;
+}
+
+lq_status_t lq_debug_launches_prefetched(const lq_cache_t* c, int64_t* n) {
+  if (!c || !n) return LQ_ERR_INVALID_ARG;
+  *n = c->n_prefetched;
   return LQ_OK;
 }
 

@@ -1,0 +1,119 @@
+"""Order on the device: what a call may assume of the work enqueued before it, on other streams, across stream captures and
+after a call that failed."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_common import assert_images_equal, attn_tolerance
+from paper_2503_19950_b200 import LQ_FLAG_OVERLAP_DECODE, LogQuantCache, LogQuantError, binding, build, synth
+
+pytestmark = pytest.mark.gpu
+B, HQ, HKV, W, G, D = 1, 8, 2, 32, 32, 128
+BUSY = 60_000_000  # clock cycles of a kernel that keeps a stream busy: about 30 ms
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+
+
+def _filled(seed, n):
+    """Keys and values of n tokens and the oracle's cache that holds them."""
+    k, v = synth.keys_values(seed, B, HKV, n, D, "cuda")
+    oc = oracle.OracleCache(B, HQ, HKV, D, W, G)
+    oc.append(synth.bf16_bits(k), synth.bf16_bits(v))
+    return k, v, oc
+
+
+def _check_attention(oc, q, out):
+    ref = oc.attention(synth.bf16_bits(q), 1 / np.sqrt(D))
+    assert np.abs(out.cpu().numpy() - ref).max() <= attn_tolerance(ref)
+
+
+def _two_layers(flags=0):
+    """A cache of two small layers with a few steps behind them, and the calls of further steps."""
+    cache = LogQuantCache(2, B, HQ, HKV, W, G, max_tokens=256, flags=flags)
+    q, out = synth.queries(4, B, HQ, D, 0, "cuda"), torch.empty(B, HQ, D, device="cuda")
+    k, v, _ = _filled(4, 150)
+    row = tuple(x[:, :, :1].contiguous() for x in (k, v))
+    for layer in range(2):
+        cache.append(layer, k, v)
+
+    def fused(layer):
+        cache.append_decode_attn(layer, *row, q, out)
+
+    def plain(layer):
+        cache.decode_attn(layer, q, out)
+
+    torch.cuda.synchronize()
+    return cache, fused, plain
+
+
+def test_which_launches_fetch_their_stages_early():
+    """Default flags, small launches: one that follows a decode launch of the same cache and stream, unless that one wrote
+    a row of the same layer."""
+    cache, fused, plain = _two_layers()
+    other = torch.cuda.Stream()
+    count = [cache.debug_launches_prefetched()]
+
+    def early(call, layer):
+        call(layer)
+        count.append(cache.debug_launches_prefetched())
+        return count[-1] - count[-2]
+
+    assert early(plain, 0) == 0      # behind the appends
+    assert early(plain, 0) == 1
+    assert early(plain, 1) == 1
+    assert early(fused, 0) == 1
+    assert early(plain, 0) == 0      # behind the launch that wrote its row
+    assert early(plain, 1) == 1
+    assert early(fused, 0) == 1
+    assert early(plain, 1) == 1
+    assert early(plain, 0) == 1      # that launch has waited for the one that wrote the row
+    other.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(other):
+        assert early(plain, 1) == 0  # another stream
+        assert early(plain, 0) == 1
+    torch.cuda.current_stream().wait_stream(other)
+    assert early(plain, 0) == 0
+    k, v, _ = _filled(5, 40)
+    cache.append(0, k, v)            # an overflow step on the way
+    assert early(plain, 1) == 0
+    cache.profile_enable()
+    assert early(plain, 0) == 0      # timed launches start alone
+    cache.profile_enable(False)
+    assert early(plain, 0) == 0
+    assert early(plain, 1) == 1
+    torch.cuda.synchronize()
+    assert cache.kernel_status() == 0
+    cache.close()
+
+
+def test_a_launch_that_failed_was_not_there():
+    """A decode call that returns an error has launched nothing: the call after it must not take it for the launch that
+    stands between it and the one that wrote its row."""
+    from cuda.bindings import runtime
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        cache, fused, plain = _two_layers()
+        plain(1)
+        fused(0)
+        handle = runtime.cudaStream_t(stream.cuda_stream)
+        # a capture that a forbidden synchronisation has made invalid: every launch on the stream fails until it is ended
+        assert runtime.cudaStreamBeginCapture(handle, runtime.cudaStreamCaptureMode.cudaStreamCaptureModeThreadLocal)[0] == 0
+        assert runtime.cudaStreamSynchronize(handle)[0] != 0
+        with pytest.raises(LogQuantError) as err:
+            plain(1)
+        assert err.value.status == binding.LQ_ERR_CUDA
+        assert runtime.cudaStreamEndCapture(handle)[0] != 0
+        runtime.cudaGetLastError()
+        before = cache.debug_launches_prefetched()
+        plain(0)
+        assert cache.debug_launches_prefetched() == before
+        k, v, _ = _filled(5, 1)
+        cache.append(1, k, v)        # the error of the earlier call is not reported again
+        plain(1)
+    torch.cuda.synchronize()
+    assert cache.kernel_status() == 0
+    cache.close()
