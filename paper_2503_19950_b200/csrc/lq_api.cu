@@ -76,6 +76,7 @@ struct lq_cache {
   int last_decode_layer = -1;
   int last_row_layer = -1;  // layer to which that launch appended a row (-1: none)
   cudaStream_t last_decode_stream = nullptr;
+  unsigned long long last_decode_capture = 0;  // the stream capture that launch was recorded in (capture_id)
   // Rows written by fused append+attention launches that may still be running.  An overlapped launch of the same
   // layer reads that row in its main loop, before its dependency wait, so it may overlap only when the writing
   // launch A is known to be complete.  Known without asking the device: a CTA of these kernels leaves only after
@@ -118,6 +119,19 @@ lq_status_t cuda_fail(lq_cache* c, cudaError_t e, const char* what) {
   if (c) c->last_error = buf;
   cudaGetLastError();  // (else the next launch that asks for its error would be told of this one)
   return LQ_ERR_CUDA;
+}
+
+// The capture that `st` is recording: its id, 0 for none (launches run), kCaptureUnknown when the runtime will not say.  A
+// captured launch runs when its graph does, so it is no predecessor of a launch outside that capture.
+constexpr unsigned long long kCaptureUnknown = ~0ull;
+unsigned long long capture_id(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return kCaptureUnknown;
+  }
+  return status == cudaStreamCaptureStatusNone ? 0 : status == cudaStreamCaptureStatusActive ? id : kCaptureUnknown;
 }
 
 // Every device block of a cache -- long-lived or temporary -- comes from here: the caller's allocator when one
@@ -1070,8 +1084,11 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
     // twice the CTAs of these kernels the device can hold (51 KB of shared memory each: at most four per SM)
     const int64_t resident_bound = 2LL * max_ctas_decode_mma(c->sm_count);
     const bool row_safe = c->row_mark[layer] < 0 || c->ctas_since_wait - c->row_mark[layer] >= resident_bound;
-    a.early = (c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) && !timed && c->last_decode_layer >= 0 &&
-              c->last_decode_layer != layer && c->last_decode_stream == st && row_safe;
+    // this cache's last work was a decode launch on this stream, both of them eager or both part of one capture
+    const unsigned long long capture = capture_id(st);
+    const bool follows = c->last_decode_layer >= 0 && c->last_decode_stream == st && c->last_decode_capture == capture &&
+                         capture != kCaptureUnknown;
+    a.early = (c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) && !timed && follows && c->last_decode_layer != layer && row_safe;
     plan_decode_mma(a, c->sm_count, c->max_splits, c->cfg.n_splits);
     if (a.rowinfo) {
       a.S = a.early ? c->pad_stride_ov[layer] : c->pad_stride[layer];
@@ -1082,11 +1099,10 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
       }
       a.n_extra = 0;
     }
-    // A small launch may read its stores before it waits for the launch before it, if that was this cache's last work, a
-    // decode launch on the same stream (so that everything older has finished: it waited at entry itself) and did not write
-    // a row of this layer.
+    // A small launch may read its stores before it waits for the launch before it, if that was a decode launch of this cache
+    // (so that everything older has finished: it waited at entry itself) and did not write a row of this layer.
     if (a.rowinfo || (c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) || timed) a.small = 0;
-    a.prefetch = a.small && c->last_decode_layer >= 0 && c->last_row_layer != layer && c->last_decode_stream == st;
+    a.prefetch = a.small && follows && c->last_row_layer != layer;
     a.tickets = c->tickets;  // the CTA that completes a (b, kv) pair merges it: no second launch
     a.acc = c->acc;
     // (a launch that fails is none: the next one derives nothing from it, nor from the one before it)
@@ -1100,6 +1116,7 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
     c->ctas_since_wait += a.rowinfo ? a.n_ctas : c->cfg.batch * c->cfg.n_kv_heads * (a.S - 1) + a.n_extra;  // the grid
     c->row_mark[layer] = new_k != nullptr ? c->ctas_since_wait : -1;
     c->last_row_layer = new_k != nullptr ? layer : -1;
+    c->last_decode_capture = capture;
     if (a.early) c->n_overlapped++;
     if (a.prefetch) c->n_prefetched++;
   } else if (use_umma(c)) {

@@ -117,3 +117,29 @@ def test_a_launch_that_failed_was_not_there():
     torch.cuda.synchronize()
     assert cache.kernel_status() == 0
     cache.close()
+
+
+def test_captured_launches_are_no_predecessors_of_eager_ones():
+    """A captured launch has not run: neither the early fetch nor the overlapped form may be derived from it."""
+    stream = torch.cuda.Stream()
+    for flags, count in ((0, lambda c: c.debug_launches_prefetched()), (LQ_FLAG_OVERLAP_DECODE, lambda c: c.info(0).n_launches_overlapped)):
+        with torch.cuda.stream(stream):
+            cache, fused, plain = _two_layers(flags)
+            plain(1)
+            fused(0)
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                before = count(cache)
+                plain(1)             # follows nothing that is part of the graph
+                assert count(cache) == before
+                plain(1)
+            before = count(cache)
+            plain(0)
+            assert count(cache) == before
+            plain(1)
+            assert count(cache) == before + 1
+            graph.replay()
+        torch.cuda.synchronize()
+        assert cache.kernel_status() == 0
+        del graph
+        cache.close()
