@@ -107,7 +107,8 @@ typedef struct {
   int32_t flags;         /* LQ_FLAG_* bits, 0 = none                                             */
   /* Optional device allocator (all three NULL / 0: cudaMalloc and cudaFree).  dev_alloc returns device memory of
      at least `bytes` bytes, 256-byte aligned, on `device`, or NULL on failure (the call that needed it then gives
-     LQ_ERR_OOM); every block is handed back to dev_free by lq_destroy (or at once when creation fails).  Both
+     LQ_ERR_OOM); every block is handed back to dev_free by lq_destroy (or at once when creation fails).  Work still
+     enqueued may use a block that is handed out, if it is on the stream lq_cache_create_on_stream names.  Both
      are called on the host, from the thread that calls into the library, with alloc_ctx passed through. */
   void* (*dev_alloc)(size_t bytes, void* alloc_ctx);
   void (*dev_free)(void* ptr, void* alloc_ctx);
@@ -162,8 +163,16 @@ typedef struct {
 /* Create a cache.  Validates the configuration (LQ_ERR_INVALID_ARG / LQ_ERR_UNSUPPORTED),
  * selects cfg->device and allocates both stores and the split-K workspace with cudaMalloc
  * (LQ_ERR_OOM).  *out is written only on success.  (Problem statement: window W of Sec. 2.5,
- * group size G and INT2 of Sec. 3.1.) */
+ * group size G and INT2 of Sec. 3.1.)  Nothing is enqueued: what the library writes to a new block before its first
+ * use (zeros, guard bytes) goes out on the stream of the first call that enqueues work on the cache -- if that
+ * stream is being captured, beside the capture and before the call returns.  The same holds for the block that
+ * lq_set_padding allocates. */
 lq_status_t lq_cache_create(const lq_config_t* cfg, lq_cache_t** out);
+
+/* lq_cache_create for a dev_alloc whose blocks are free in the order of `alloc_stream`, i.e. may still be in use by
+ * work enqueued there before the allocation: the first writes to a block wait for that work, whichever stream they
+ * go out on.  lq_cache_create takes the legacy default stream for it.  Without dev_alloc the two are the same. */
+lq_status_t lq_cache_create_on_stream(const lq_config_t* cfg, void* alloc_stream, lq_cache_t** out);
 
 /* Free the cache and its device memory.  NULL is a no-op.  The caller must have synchronised
  * every stream that still has work of this cache in flight. */

@@ -50,7 +50,7 @@ class lq_device_image_t(C.Structure):
                [(n, C.c_void_p) for n in ("fp_k", "fp_v", "k_codes", "v_codes", "k_scale", "k_zero", "v_scale", "v_zero")]
 
 
-SYMBOLS = ["lq_cache_create", "lq_destroy", "lq_append", "lq_compress", "lq_decode_attn", "lq_append_decode_attn",
+SYMBOLS = ["lq_cache_create", "lq_cache_create_on_stream", "lq_destroy", "lq_append", "lq_compress", "lq_decode_attn", "lq_append_decode_attn",
            "lq_decode_attn_fp_only", "lq_set_padding",
            "lq_decode_step_host", "lq_profile_enable", "lq_profile_read", "lq_kernel_status", "lq_cache_info", "lq_export",
            "lq_next_evicted_ids", "lq_decode_attn_image_static", "lq_status_str", "lq_last_error", "lq_check_guards",
@@ -76,6 +76,7 @@ def load_library():
         L = C.CDLL(_LIB_PATH)
         vp, i32 = C.c_void_p, C.c_int32
         L.lq_cache_create.argtypes = [C.POINTER(lq_config_t), C.POINTER(vp)]
+        L.lq_cache_create_on_stream.argtypes = [C.POINTER(lq_config_t), vp, C.POINTER(vp)]
         L.lq_destroy.argtypes = [vp]
         L.lq_append.argtypes = [vp, i32, vp, vp, i32, vp]
         L.lq_compress.argtypes = [vp, i32, vp]
@@ -173,8 +174,9 @@ class LogQuantCache:
     def __init__(self, n_layers, batch, n_q_heads, n_kv_heads, window, group, max_tokens, head_dim=128, bits=2,
                  auto_compress=True, device=0, kernel=LQ_KERNEL_AUTO, n_splits=0, filter=0, allocator=None, flags=0):
         """allocator: None (cudaMalloc / cudaFree), "torch" (every device block of the cache is a uint8 tensor from
-        torch's caching allocator, kept alive until the cache is closed), or a pair of callables
-        (alloc(bytes) -> device address or 0, free(address))."""
+        torch's caching allocator, drawn from the pool of the stream that is current now and kept alive until the cache
+        is closed), or a pair of callables (alloc(bytes) -> device address or 0, free(address)), whose blocks must be
+        free in the order of the legacy default stream."""
         self._lib = load_library()
         # the calls of a decode step, bound once
         self._append_decode_attn, self._decode_attn = self._lib.lq_append_decode_attn, self._lib.lq_decode_attn
@@ -182,12 +184,22 @@ class LogQuantCache:
         self._blocks = {}
         LogQuantCache.live.add(self)
         alloc_cb, free_cb = ALLOC_FN(0), FREE_FN(0)
+        pool = None  # handle of the stream whose pool the blocks come from
         if allocator == "torch":
             import torch
+            raw_stream, pool_stream, where = torch._C._cuda_getCurrentRawStream, None, None
+            if device >= 0 and (torch.cuda.is_initialized() or torch.cuda.is_available()):
+                torch.cuda.init()
+                pool, where = raw_stream(device), torch.device("cuda", device)
+                pool_stream = torch.cuda.current_stream(device) if pool else None  # None: the default stream
 
             def _alloc(nbytes, _ctx):
                 try:
-                    t = torch.empty(max(int(nbytes), 1), dtype=torch.uint8, device=torch.device("cuda", device))
+                    if raw_stream(device) == pool:
+                        t = torch.empty(nbytes, dtype=torch.uint8, device=where)
+                    else:
+                        with torch.cuda.stream(pool_stream or torch.cuda.default_stream(device)):
+                            t = torch.empty(nbytes, dtype=torch.uint8, device=where)
                 except RuntimeError:
                     return 0
                 self._blocks[t.data_ptr()] = t
@@ -205,7 +217,7 @@ class LogQuantCache:
         self.cfg = lq_config_t(n_layers, batch, n_q_heads, n_kv_heads, head_dim, window, group, bits, max_tokens,
                                int(auto_compress), device, kernel, n_splits, filter, flags, alloc_cb, free_cb, None)
         self._h = C.c_void_p()
-        self._check(self._lib.lq_cache_create(C.byref(self.cfg), C.byref(self._h)), create=True)
+        self._check(self._lib.lq_cache_create_on_stream(C.byref(self.cfg), pool, C.byref(self._h)), create=True)
 
     def _check(self, status, create=False):
         if status != LQ_OK:

@@ -109,6 +109,15 @@ struct lq_cache {
   size_t ev_used = 0;
   std::string last_error;
   std::vector<std::pair<uint8_t*, int64_t>> blocks;  // device blocks (address, payload bytes): guard bytes follow the payload
+  // What the library writes to new blocks before anything else (guard bytes, zeros): enqueued by the first call that enqueues
+  // work, on that call's stream, so that no stream sees a block before it is written (first_writes).
+  BlockInit init = {};
+  bool init_pending = false, zero_fp = false;
+  // With the caller's allocator: blocks are free in the order of alloc_stream, of which alloc_event marks the place of the
+  // newest one (valid with alloc_marked).
+  cudaStream_t alloc_stream = nullptr;
+  cudaEvent_t alloc_event = nullptr;
+  bool alloc_marked = false;
 };
 
 namespace {
@@ -125,6 +134,7 @@ lq_status_t cuda_fail(lq_cache* c, cudaError_t e, const char* what) {
 // captured launch runs when its graph does, so it is no predecessor of a launch outside that capture.
 constexpr unsigned long long kCaptureUnknown = ~0ull;
 unsigned long long capture_id(cudaStream_t st) {
+  if (st == nullptr) return 0;  // the legacy default stream cannot be captured
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
   unsigned long long id = 0;
   if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
@@ -136,8 +146,8 @@ unsigned long long capture_id(cudaStream_t st) {
 
 // Every device block of a cache -- long-lived or temporary -- comes from here: the caller's allocator when one
 // is set, else cudaMalloc.  `bytes` is rounded up to 256 so that the guard starts on an aligned address.
-// guard = false: the caller fills the guard bytes in (launch_init_blocks).
-bool dev_alloc(lq_cache* c, void** p, int64_t bytes, bool temporary = false, bool guard = true) {
+// The guard bytes of a long-lived block are left to first_writes; a temporary one is asked for while the device is idle.
+bool dev_alloc(lq_cache* c, void** p, int64_t bytes, bool temporary = false) {
   const int64_t payload = (bytes + 255) / 256 * 256, total = payload + kGuardBytes;
   if (c->cfg.dev_alloc) {  // the caller's allocator
     *p = c->cfg.dev_alloc(static_cast<size_t>(total), c->cfg.alloc_ctx);
@@ -147,10 +157,70 @@ bool dev_alloc(lq_cache* c, void** p, int64_t bytes, bool temporary = false, boo
     *p = nullptr;
     return false;
   }
-  if (guard && cudaMemset(static_cast<uint8_t*>(*p) + payload, kGuardPattern, kGuardBytes) != cudaSuccess) cudaGetLastError();
+  uint8_t* guard = static_cast<uint8_t*>(*p) + payload;
+  if (temporary) {
+    if (cudaMemset(guard, kGuardPattern, kGuardBytes) != cudaSuccess) cudaGetLastError();
+  } else {
+    c->init.guard[c->init.n_guards++] = guard;
+    c->init_pending = true;
+  }
   c->blocks.emplace_back(static_cast<uint8_t*>(*p), payload);
   if (!temporary) c->bytes_device += total;
   return true;
+}
+
+// To be called behind the allocation of long-lived blocks: marks the place in alloc_stream from which on they are free.
+bool mark_allocations(lq_cache* c) {
+  // (memory from an allocator that takes part in a capture belongs to the graph: nothing pending uses it)
+  if (c->cfg.dev_alloc == nullptr || capture_id(c->alloc_stream) != 0) return true;
+  cudaError_t e = cudaSuccess;
+  if (c->alloc_event == nullptr) e = cudaEventCreateWithFlags(&c->alloc_event, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(c->alloc_event, c->alloc_stream);
+  c->alloc_marked |= e == cudaSuccess;
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess;
+}
+
+// Writes new blocks before the caller enqueues their first use on `st`.
+lq_status_t first_writes(lq_cache* c, cudaStream_t st) {
+  if (!c->init_pending) return LQ_OK;
+  // in a capture the writes would run with every replay: they run now, on a stream of their own, before the call returns
+  const bool aside = capture_id(st) != 0;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaStream_t on = st;
+  cudaError_t e = cudaSuccess;
+  if (aside) {
+    e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return cuda_fail(c, e, "cudaThreadExchangeStreamCaptureMode");
+    e = cudaStreamCreateWithFlags(&on, cudaStreamNonBlocking);
+    if (e != cudaSuccess) on = nullptr;
+  }
+  if (e == cudaSuccess && c->alloc_marked && on != c->alloc_stream) e = cudaStreamWaitEvent(on, c->alloc_event, 0);
+  if (e == cudaSuccess) e = launch_init_blocks(c->init, on);
+  // the fp store must never hold non-finite garbage in unused slots of a partly filled tile
+  if (e == cudaSuccess && c->zero_fp)
+    e = cudaMemsetAsync(c->cv.fp, 0, static_cast<size_t>(c->cv.fp_layer_stride) * c->cfg.n_layers, on);
+  if (aside) {
+    if (e == cudaSuccess) e = cudaStreamSynchronize(on);
+    if (on) cudaStreamDestroy(on);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  if (e != cudaSuccess) return cuda_fail(c, e, "first writes to the device blocks");
+  c->init = {};
+  c->init_pending = c->zero_fp = c->alloc_marked = false;
+  c->last_decode_layer = -1;
+  return LQ_OK;
+}
+
+// The same for a call that synchronises the device.
+lq_status_t first_writes_now(lq_cache* c) {
+  if (!c->init_pending) return LQ_OK;
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) return cuda_fail(c, e, "cudaDeviceSynchronize");
+  const lq_status_t s = first_writes(c, nullptr);
+  if (s != LQ_OK) return s;
+  e = cudaDeviceSynchronize();
+  return e == cudaSuccess ? LQ_OK : cuda_fail(c, e, "cudaDeviceSynchronize");
 }
 
 void dev_release(lq_cache* c, void* p) {
@@ -191,6 +261,7 @@ void free_all(lq_cache* c) {
     dev_release(c, c->stage_out);
     dev_release(c, c->masks);
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
+    if (c->alloc_event) cudaEventDestroy(c->alloc_event);
   }
 }
 
@@ -477,6 +548,10 @@ const char* lq_status_str(lq_status_t s) {
 const char* lq_last_error(const lq_cache_t* c) { return c ? c->last_error.c_str() : ""; }
 
 lq_status_t lq_cache_create(const lq_config_t* cfg, lq_cache_t** out) {
+  return lq_cache_create_on_stream(cfg, nullptr, out);
+}
+
+lq_status_t lq_cache_create_on_stream(const lq_config_t* cfg, void* alloc_stream, lq_cache_t** out) {
   if (!cfg || !out) return LQ_ERR_INVALID_ARG;
   if (cfg->n_layers < 1 || cfg->batch < 1 || cfg->n_q_heads < 1 || cfg->n_kv_heads < 1 ||
       cfg->window < 1 || cfg->group < 1 || cfg->max_tokens < 1 || cfg->n_splits < 0)
@@ -494,6 +569,7 @@ lq_status_t lq_cache_create(const lq_config_t* cfg, lq_cache_t** out) {
   lq_cache* c = new (std::nothrow) lq_cache;
   if (!c) return LQ_ERR_OOM;
   c->cfg = *cfg;
+  c->alloc_stream = static_cast<cudaStream_t>(alloc_stream);
   c->dry = cfg->device == LQ_DEVICE_NONE;
   const int W = cfg->window, G = cfg->group;
   const int64_t pairs = static_cast<int64_t>(cfg->batch) * cfg->n_kv_heads;
@@ -526,17 +602,15 @@ lq_status_t lq_cache_create(const lq_config_t* cfg, lq_cache_t** out) {
     const int r = ratio(c);
     const int64_t q_bytes = static_cast<int64_t>(cfg->n_layers) * cfg->batch * cfg->n_q_heads * kD * 2;
     const int64_t acc_bytes = static_cast<int64_t>(pairs) * kAccStride * 4;
-    auto alloc = [&](auto** p, int64_t bytes) { return dev_alloc(c, reinterpret_cast<void**>(p), bytes, false, false); };
+    auto alloc = [&](auto** p, int64_t bytes) { return dev_alloc(c, reinterpret_cast<void**>(p), bytes); };
     bool ok = alloc(&cv.quant, cv.quant_layer_stride * cfg->n_layers) && alloc(&cv.fp, cv.fp_layer_stride * cfg->n_layers) &&
               alloc(&c->part_o, pairs * c->max_splits * r * kD * 4) && alloc(&c->part_ml, pairs * c->max_splits * r * 2 * 4) &&
               alloc(&c->status, 256) && alloc(&c->tickets, pairs * 128) && alloc(&c->acc, acc_bytes) &&
               alloc(&c->ingest_idx, ingest_idx_ints(c) * 4) && alloc(&c->stage_k, cfg->n_layers * pairs * kD * 2) &&
-              alloc(&c->stage_v, cfg->n_layers * pairs * kD * 2) && alloc(&c->stage_q, q_bytes) && alloc(&c->stage_out, 2 * q_bytes);
+              alloc(&c->stage_v, cfg->n_layers * pairs * kD * 2) && alloc(&c->stage_q, q_bytes) && alloc(&c->stage_out, 2 * q_bytes) && mark_allocations(c);
     cv.status = c->status;
     if (ok) {
-      BlockInit init;
-      std::memset(&init, 0, sizeof init);
-      for (const auto& blk : c->blocks) init.guard[init.n_guards++] = blk.first + blk.second;
+      BlockInit& init = c->init;
       auto zero = [&](void* p, int64_t bytes) {
         init.zero[init.n_zero] = static_cast<uint4*>(p);
         init.zero_chunks[init.n_zero++] = bytes / 16;
@@ -544,11 +618,8 @@ lq_status_t lq_cache_create(const lq_config_t* cfg, lq_cache_t** out) {
       zero(c->status, 256);
       zero(c->tickets, pairs * 128);
       zero(c->acc, acc_bytes);
-      ok = launch_init_blocks(init, nullptr) == cudaSuccess;
-    }
-    // the fp store must never hold non-finite garbage in unused slots of a partly filled tile
-    if (ok) ok = cudaMemset(cv.fp, 0, static_cast<size_t>(cv.fp_layer_stride) * cfg->n_layers) == cudaSuccess;
-    if (!ok) {
+      c->zero_fp = true;
+    } else {
       free_all(c);
       delete c;
       cudaGetLastError();
@@ -885,6 +956,8 @@ lq_status_t append_impl(lq_cache_t* c, int32_t layer, const void* k, const void*
   if (L.n_seen + n > c->cfg.max_tokens) return LQ_ERR_CAPACITY;
   if (!c->cfg.auto_compress && kept(L) + n > 3 * W) return LQ_ERR_WINDOW_FULL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const lq_status_t ready = first_writes(c, st);
+  if (ready != LQ_OK) return ready;
   // more than one launch's worth of work: a prompt for an empty layer, or a chunk of at least two windows that makes
   // a layer already in use overflow.  Below two windows the index upload of the one-launch path costs more than the
   // launches it saves.
@@ -932,6 +1005,8 @@ lq_status_t lq_compress(lq_cache_t* c, int32_t layer, void* stream) {
       if (kept(c->layers[i]) == 3 * W) full.push_back(i);
   }
   if (full.empty()) return LQ_OK;
+  const lq_status_t ready = first_writes(c, static_cast<cudaStream_t>(stream));
+  if (ready != LQ_OK) return ready;
   return run_events(c, full, static_cast<cudaStream_t>(stream));
 }
 
@@ -966,7 +1041,8 @@ lq_status_t lq_set_padding(lq_cache_t* c, const int32_t* pad_host) {
     c->q_words = static_cast<int>((c->cfg.max_tokens + 31) / 32);
     c->map_words = std::max(max_ctas_decode_mma(c->sm_count), B * c->cfg.n_kv_heads);  // at least one CTA per pair
     c->mask_layer_words = static_cast<int64_t>(B) * (4 + c->fp_words + c->q_words) + 2 * (B * c->cfg.n_kv_heads + c->map_words);
-    if (!dev_alloc(c, reinterpret_cast<void**>(&c->masks), c->mask_layer_words * c->cfg.n_layers * 4)) return LQ_ERR_OOM;
+    if (!dev_alloc(c, reinterpret_cast<void**>(&c->masks), c->mask_layer_words * c->cfg.n_layers * 4) || !mark_allocations(c))
+      return LQ_ERR_OOM;
   }
   c->pad.assign(pad_host, pad_host + B);
   c->has_pad = false;
@@ -1029,6 +1105,8 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
   LayerState& L = c->layers[layer];
   if (L.n_fp + L.n_quant == 0) return LQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const lq_status_t ready = first_writes(c, st);
+  if (ready != LQ_OK) return ready;
   DecodeArgs a;
   a.cv = c->cv;
   a.layer = layer;
@@ -1159,6 +1237,8 @@ lq_status_t lq_decode_step_host(lq_cache_t* c, int32_t layer, const void* k_host
   uint8_t* sv = c->stage_v + layer * kvb;
   uint8_t* sq = c->stage_q + layer * qb;
   uint8_t* so = c->stage_out + layer * qb * 2;
+  const lq_status_t ready = first_writes(c, st);
+  if (ready != LQ_OK) return ready;
   cudaError_t e;
   // Page-locked host buffers that the device can address are used in place, by the same single launch as the
   // device-buffer step (lq_append_decode_attn): the attention kernel takes the new k and v rows and the query
@@ -1239,6 +1319,8 @@ lq_status_t lq_kernel_status(lq_cache_t* c, int32_t* word) {
   if (!c || !word) return LQ_ERR_INVALID_ARG;
   *word = 0;
   if (c->dry) return LQ_OK;
+  const lq_status_t ready = first_writes_now(c);
+  if (ready != LQ_OK) return ready;
   cudaError_t e = cudaMemcpy(word, c->status, sizeof(int32_t), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(c, e, "status read");
   return LQ_OK;
@@ -1247,6 +1329,8 @@ lq_status_t lq_kernel_status(lq_cache_t* c, int32_t* word) {
 lq_status_t lq_reset_kernel_status(lq_cache_t* c) {
   if (!c) return LQ_ERR_INVALID_ARG;
   if (c->dry) return LQ_OK;
+  const lq_status_t ready = first_writes_now(c);
+  if (ready != LQ_OK) return ready;
   cudaError_t e = cudaDeviceSynchronize();
   if (e == cudaSuccess) e = cudaMemset(c->status, 0, sizeof(int32_t));
   if (e != cudaSuccess) return cuda_fail(c, e, "status reset");
@@ -1429,6 +1513,7 @@ lq_status_t lq_import(lq_cache_t* c, int32_t layer, const lq_image_t* img, int64
   lq_status_t status = LQ_OK;
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) status = cuda_fail(c, e, "cudaDeviceSynchronize");
+  if (status == LQ_OK) status = first_writes_now(c);
   for (auto& b : bufs) {
     if (status != LQ_OK || b.bytes == 0) continue;
     if (!dev_alloc(c, &b.dev, b.bytes, true)) status = LQ_ERR_OOM;
@@ -1464,6 +1549,8 @@ lq_status_t lq_check_guards(lq_cache_t* c, int32_t* n_damaged) {
   if (!c || !n_damaged) return LQ_ERR_INVALID_ARG;
   *n_damaged = 0;
   if (c->dry) return LQ_OK;
+  const lq_status_t ready = first_writes_now(c);
+  if (ready != LQ_OK) return ready;
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaDeviceSynchronize");
   *n_damaged = damaged_guards(c);

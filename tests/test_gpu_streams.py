@@ -31,6 +31,80 @@ def _check_attention(oc, q, out):
     assert np.abs(out.cpu().numpy() - ref).max() <= attn_tolerance(ref)
 
 
+@pytest.mark.parametrize("allocator", [None, "torch"])
+def test_a_new_cache_on_another_stream_than_the_busy_default_one(allocator):
+    """The zeros of a new cache come before its first tokens whatever the default stream is doing."""
+    k, v, oc = _filled(1, 200)
+    q, out = synth.queries(1, B, HQ, D, 0, "cuda"), torch.full((B, HQ, D), float("nan"), device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(BUSY)
+    cache = LogQuantCache(1, B, HQ, HKV, W, G, max_tokens=256, allocator=allocator)
+    cache.append(0, k, v, stream=side)
+    cache.decode_attn(0, q, out, stream=side)
+    side.synchronize()
+    torch.cuda.synchronize()
+    assert_images_equal(cache.export(0), oc.export())
+    _check_attention(oc, q, out)
+    assert cache.kernel_status() == 0
+    cache.close()
+
+
+def test_blocks_of_a_new_cache_that_the_stream_still_uses():
+    """torch hands a freed block out again while kernels of its stream still read it: nothing may be written to it outside
+    that stream's order, neither by the creation of a cache nor by its first padding."""
+    k, v, oc = _filled(2, 200)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def new_cache():
+        cache = LogQuantCache(1, B, HQ, HKV, W, G, max_tokens=256, allocator="torch")
+        cache.set_padding([3])
+        return cache
+
+    with torch.cuda.stream(side):
+        first = new_cache()
+        sizes = [t.numel() for t in first._blocks.values()]
+        first.close()
+        side.synchronize()
+        old = [torch.full((n,), 7, dtype=torch.uint8, device="cuda") for n in sizes]
+        read = [torch.empty_like(x) for x in old]
+        at = {x.data_ptr() for x in old}
+        torch.cuda._sleep(BUSY)
+        for x, y in zip(old, read):
+            y.copy_(x)
+        del old, x
+        cache = new_cache()
+        assert at & set(cache._blocks), "no block was handed out again: the test shows nothing"
+        cache.append(0, k, v)
+    torch.cuda.synchronize()
+    assert all(bool((y == 7).all()) for y in read)
+    assert_images_equal(cache.export(0), oc.export())
+    cache.close()
+
+
+@pytest.mark.parametrize("allocator", [None, "torch"])
+def test_a_new_cache_whose_first_calls_are_captured(allocator):
+    """The zeros of a new cache are no part of a graph: they are there before its first replay and do not come again."""
+    k, v, oc = _filled(3, 2)
+    q, out = synth.queries(3, B, HQ, D, 0, "cuda"), torch.full((B, HQ, D), float("nan"), device="cuda")
+    rows = [tuple(x[:, :, t:t + 1].contiguous() for x in (k, v)) for t in range(2)]
+    torch.cuda.synchronize()
+    cache = LogQuantCache(1, B, HQ, HKV, W, G, max_tokens=256, allocator=allocator)
+    graphs = [torch.cuda.CUDAGraph() for _ in rows]
+    for g, row in zip(graphs, rows):
+        with torch.cuda.graph(g):
+            cache.append(0, *row)
+            cache.decode_attn(0, q, out)
+    for g in (graphs[0], graphs[1], graphs[1], graphs[0], graphs[1]):
+        g.replay()
+    torch.cuda.synchronize()
+    assert_images_equal(cache.export(0), oc.export())
+    _check_attention(oc, q, out)
+    assert cache.kernel_status() == 0 and cache.check_guards() == 0
+    cache.close()
+
+
 def _two_layers(flags=0):
     """A cache of two small layers with a few steps behind them, and the calls of further steps."""
     cache = LogQuantCache(2, B, HQ, HKV, W, G, max_tokens=256, flags=flags)
