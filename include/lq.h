@@ -185,8 +185,10 @@ lq_status_t lq_destroy(lq_cache_t* cache);
  * when the layer is still empty and n_tokens > 3W (a prompt), or the layer is in use, n_tokens >= 2W
  * and the window overflows on the way (a chunk of a prompt), the same
  * result -- the same image -- is produced by one kernel launch from the kept/removed sets that
- * Algorithm 1 fixes in advance (the index lists of that launch are copied from pageable host memory
- * on `stream`; calls that ingest prompts must share one stream or be ordered by the caller). */
+ * Algorithm 1 fixes in advance.  The index lists of that launch are copied from pageable host memory on
+ * `stream` by the first layer that needs them; layers in the same state that follow on the stream share them
+ * (calls that ingest prompts must share one stream or be ordered by the caller).  A call on a stream that is
+ * being captured takes the split form instead. */
 lq_status_t lq_append(lq_cache_t* cache, int32_t layer, const void* k, const void* v,
                       int32_t n_tokens, void* stream);
 

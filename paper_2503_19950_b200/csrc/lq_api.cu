@@ -758,23 +758,18 @@ void copy_bookkeeping(LayerState& to, const LayerState& from) {  // all but quan
   to.age_slot = from.age_slot; to.pend_slot = from.pend_slot; to.slot_token = from.slot_token;
 }
 
-// Index lists of a plan on the device, ready for a kernel on `st`.  Lists uploaded on this very stream are there already;
-// a stream that is being captured neither finds nor leaves any (its copy runs when the graph does).
+// Index lists of a plan on the device, ready for a kernel on `st` (which is not being captured).  Lists uploaded on this very
+// stream are there already.
 lq_status_t launch_plan(lq_cache* c, int layer, IngestPlan& p, const int32_t* idx, const void* k, const void* v, cudaStream_t st) {
-  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   unsigned long long id = 0;
-  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || cudaStreamGetId(st, &id) != cudaSuccess) {
-    cudaGetLastError();
-    capture = cudaStreamCaptureStatusActive;
-  }
-  const bool plain = capture == cudaStreamCaptureStatusNone;
-  cudaError_t e;
-  if (!(plain && p.uploaded && p.uploaded_on == id)) {
+  cudaError_t e = cudaStreamGetId(st, &id);
+  if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamGetId");
+  if (!(p.uploaded && p.uploaded_on == id)) {
     if (!idx) return LQ_ERR_UNSUPPORTED;  // (the caller makes the lists again)
     // pageable source: the runtime stages it before the call returns, so `idx` may die here
     e = cudaMemcpyAsync(c->ingest_idx + p.idx_at, idx, p.idx_ints * sizeof(int32_t), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "prompt index upload");
-    p.uploaded = plain;
+    p.uploaded = true;
     p.uploaded_on = id;
   }
   e = launch_ingest(c->cv, layer, k, v, p.n, c->ingest_idx + p.idx_at, p.n_tiles, p.has_fill, p.n_copy,
@@ -960,8 +955,9 @@ lq_status_t append_impl(lq_cache_t* c, int32_t layer, const void* k, const void*
   if (ready != LQ_OK) return ready;
   // more than one launch's worth of work: a prompt for an empty layer, or a chunk of at least two windows that makes
   // a layer already in use overflow.  Below two windows the index upload of the one-launch path costs more than the
-  // launches it saves.
-  if (c->cfg.auto_compress && extra_bytes == 0 &&
+  // launches it saves.  Under capture the lists would have to stay in host and device memory for as long as the graph does;
+  // the launches below carry everything in their arguments.
+  if (c->cfg.auto_compress && extra_bytes == 0 && (c->dry || capture_id(st) == 0) &&
       (L.n_seen == 0 ? n > 3 * W : (n >= 2 * W && kept(L) + n > 3 * W)))
     return ingest_prompt(c, layer, k, v, n, st);
   int done = 0;

@@ -105,6 +105,47 @@ def test_a_new_cache_whose_first_calls_are_captured(allocator):
     cache.close()
 
 
+@pytest.mark.parametrize("window,group", [(32, 32), (42, 64)])
+def test_prompts_ingested_under_capture(window, group):
+    """A graph whose replay ingests a prompt and two further chunks, into one layer between eager calls that ingest the same
+    and other chunks into its neighbours (whose index lists it must neither use nor overwrite)."""
+    chunks = [9 * window + 5, 2 * window + 7, 70]
+    n = sum(chunks)
+    cache = LogQuantCache(4, B, HQ, HKV, window, group, max_tokens=n + 64)
+    oracles, pieces = [], []
+    for layer in range(4):
+        k, v = synth.keys_values(20 + layer, B, HKV, n, D, "cuda")
+        sizes = [13] * (layer == 3) + chunks   # the last layer is in another state than the others
+        pieces.append([tuple(x[:, :, e - c:e].contiguous() for x in (k, v))
+                       for e, c in zip(np.cumsum(sizes), sizes) if e <= n])
+        oracles.append(oracle.OracleCache(B, HQ, HKV, D, window, group))
+        for piece in pieces[-1]:
+            oracles[-1].append(*(synth.bf16_bits(x) for x in piece))
+    q, out = synth.queries(21, B, HQ, D, 0, "cuda"), torch.empty(B, HQ, D, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def ingest(layer):
+        for piece in pieces[layer]:
+            cache.append(layer, *piece)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        ingest(0)
+        with torch.cuda.graph(graph, stream=stream):
+            ingest(1)
+            cache.decode_attn(1, q, out)
+        ingest(3)
+        graph.replay()
+        ingest(2)
+    torch.cuda.synchronize()
+    for layer in range(4):
+        assert_images_equal(cache.export(layer), oracles[layer].export())
+    _check_attention(oracles[1], q, out)
+    assert cache.kernel_status() == 0
+    cache.close()
+
+
 def _two_layers(flags=0):
     """A cache of two small layers with a few steps behind them, and the calls of further steps."""
     cache = LogQuantCache(2, B, HQ, HKV, W, G, max_tokens=256, flags=flags)
