@@ -1276,9 +1276,14 @@ void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_overrid
   // A serialised launch that leaves half of the slots empty is nothing but latency.  Its warps then take single tiles, up to
   // that half (one layer of 2 KV heads, 1024 tokens: 6.6 -> 5.8 us; beyond the half it costs, 8.2 -> 9.0 us for 8 KV heads,
   // 8192 tokens), and the next launch may move into the other half and fetch its stages (DecodeArgs::prefetch: 8.9 -> 8.2 us
-  // there; without free slots it costs, 13.4 -> 15.4 us at 32768 tokens).
+  // there; without free slots it costs, 13.4 -> 15.4 us at 32768 tokens).  Pairs whose records are summed in order keep
+  // that: no more than kMergeOneBatch CTAs, unless there are more without this rule (8 KV heads, 1250 to 2200 tokens: 12
+  // instead of 13 to 20 CTAs, 6.2 - 6.6 -> 6.7 - 6.9 us; the same 13 to 20 summed in order 7.0 - 7.8).
   a.small = !a.early && s_override <= 0 && 2 * S * pairs <= wave;
-  if (a.small) S = std::max(S, std::min((a.tiles_fp + a.tiles_quant + kWarps - 1) / kWarps, wave / 2 / pairs));
+  if (a.small) {
+    const int single = std::min((a.tiles_fp + a.tiles_quant + kWarps - 1) / kWarps, wave / 2 / pairs);
+    S = std::max(S, S <= kMergeOneBatch ? std::min(single, kMergeOneBatch) : single);
+  }
   S = std::min(S, max_records - 1);
   S = std::min(S, kMergeMax / r - 1);
   S = std::max(S, 1);

@@ -258,3 +258,19 @@ def test_captured_launches_are_no_predecessors_of_eager_ones():
         assert cache.kernel_status() == 0
         del graph
         cache.close()
+
+
+@pytest.mark.parametrize("r", [4, 7])
+@pytest.mark.parametrize("bits,group", [(2, 32), (4, 64)])
+def test_small_launches_at_ordinary_lengths_are_reproducible(r, bits, group):
+    """One sequence of 1100 to 2200 tokens: the partial results are summed in order, not as they arrive."""
+    for n in (1100, 1250, 1500, 1800, 2200):
+        cache = LogQuantCache(1, 1, 8 * r, 8, 128, group, max_tokens=n + 8, bits=bits)
+        k, v = synth.keys_values(n, 1, 8, n, D, "cuda")
+        cache.append(0, k, v)
+        q = synth.queries(n, 1, 8 * r, D, 0, "cuda")
+        outs = torch.empty(40, 1, 8 * r, D, device="cuda")
+        for out in outs:
+            cache.decode_attn(0, q, out)
+        assert bool((outs == outs[0]).all()), n
+        cache.close()
