@@ -261,7 +261,8 @@ lq_status_t lq_decode_step_host(lq_cache_t* cache, int32_t layer, const void* k_
 
 /* Kernel timing for benchmarks.  While enabled, every lq_decode_attn brackets its split-K
  * attention kernel with a pair of CUDA events on the call's stream (at most 8192 pairs are kept;
- * later launches are not timed).  lq_profile_read synchronises the device and returns the summed
+ * later launches are not timed).  A timed launch reads nothing before the launch before it has finished, and
+ * while timing is enabled small launches are split like large ones: what is timed is each kernel alone.  lq_profile_read synchronises the device and returns the summed
  * duration in milliseconds and the number of timed launches since profiling was enabled. */
 lq_status_t lq_profile_enable(lq_cache_t* cache, int32_t on);
 lq_status_t lq_profile_read(lq_cache_t* cache, double* total_ms, int64_t* n_launches);

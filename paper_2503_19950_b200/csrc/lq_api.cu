@@ -451,6 +451,9 @@ lq_status_t run_events(lq_cache* c, const std::vector<int>& full_layers, cudaStr
 }
 
 bool use_mma(const lq_cache* c) { return c->cfg.kernel == LQ_KERNEL_AUTO || c->cfg.kernel == LQ_KERNEL_MMA; }
+// Whether launches of this cache may take the form for small ones (DecodeArgs::small), which lets the next launch start early:
+// not where they overlap anyway, not while they are timed one by one, and not on padded batches, which have their own plan.
+bool may_be_small(const lq_cache* c) { return !(c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) && !c->profiling && !c->has_pad; }
 // the tcgen05 kernel serves a call unless the batch is padded (that goes through the plain kernel on the same layout)
 bool use_umma(const lq_cache* c) { return c->cfg.kernel == LQ_KERNEL_UMMA && !c->has_pad; }
 
@@ -1163,7 +1166,7 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
     const bool follows = c->last_decode_layer >= 0 && c->last_decode_stream == st && c->last_decode_capture == capture &&
                          capture != kCaptureUnknown;
     a.early = (c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) && !timed && follows && c->last_decode_layer != layer && row_safe;
-    plan_decode_mma(a, c->sm_count, c->max_splits, c->cfg.n_splits);
+    plan_decode_mma(a, c->sm_count, c->max_splits, c->cfg.n_splits, may_be_small(c));
     if (a.rowinfo) {
       a.S = a.early ? c->pad_stride_ov[layer] : c->pad_stride[layer];
       a.n_ctas = a.early ? c->pad_grid_ov[layer] : c->pad_grid[layer];
@@ -1175,7 +1178,6 @@ lq_status_t decode_impl(lq_cache_t* c, int32_t layer, const void* q, float sm_sc
     }
     // A small launch may read its stores before it waits for the launch before it, if that was a decode launch of this cache
     // (so that everything older has finished: it waited at entry itself) and did not write a row of this layer.
-    if (a.rowinfo || (c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) || timed) a.small = 0;
     a.prefetch = a.small && follows && c->last_row_layer != layer;
     a.tickets = c->tickets;  // the CTA that completes a (b, kv) pair merges it: no second launch
     a.acc = c->acc;
@@ -1377,12 +1379,12 @@ lq_status_t lq_cache_info(const lq_cache_t* c, int32_t layer, lq_info_t* info) {
     a.n_fp = L.n_fp;
     a.n_quant = L.n_quant;
     a.early = 0;  // the plan of a launch that does not overlap (an overlapped one uses a third of these CTAs)
-    plan_decode_mma(a, c->sm_count, c->max_splits, c->cfg.n_splits);
+    plan_decode_mma(a, c->sm_count, c->max_splits, c->cfg.n_splits, may_be_small(c));
     info->n_splits = a.S - 1;
     info->n_ctas = (a.S - 1) * c->cfg.batch * c->cfg.n_kv_heads + a.n_extra;
     if ((c->cfg.flags & LQ_FLAG_OVERLAP_DECODE) && !c->has_pad) {
       a.early = 1;
-      plan_decode_mma(a, c->sm_count, c->max_splits, c->cfg.n_splits);
+      plan_decode_mma(a, c->sm_count, c->max_splits, c->cfg.n_splits, false);
       info->n_ctas_overlapped = (a.S - 1) * c->cfg.batch * c->cfg.n_kv_heads + a.n_extra;
     }
   } else if (use_umma(c)) {

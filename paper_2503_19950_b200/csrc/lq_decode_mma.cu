@@ -1250,7 +1250,7 @@ __global__ void __launch_bounds__(kWarps * 32, ctas_per_sm(NCB, G, PL)) lq_decod
 
 }  // namespace
 
-void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_override) {
+void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_override, bool may_be_small) {
   const int pairs = a.cv.B * a.cv.Hkv;
   const int r = a.cv.Hq / a.cv.Hkv;
   a.tiles_fp = (a.n_fp + kFpTileSlots - 1) / kFpTileSlots;
@@ -1279,7 +1279,7 @@ void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_overrid
   // there; without free slots it costs, 13.4 -> 15.4 us at 32768 tokens).  Pairs whose records are summed in order keep
   // that: no more than kMergeOneBatch CTAs, unless there are more without this rule (8 KV heads, 1250 to 2200 tokens: 12
   // instead of 13 to 20 CTAs, 6.2 - 6.6 -> 6.7 - 6.9 us; the same 13 to 20 summed in order 7.0 - 7.8).
-  a.small = !a.early && s_override <= 0 && 2 * S * pairs <= wave;
+  a.small = may_be_small && !a.early && s_override <= 0 && 2 * S * pairs <= wave;
   if (a.small) {
     const int single = std::min((a.tiles_fp + a.tiles_quant + kWarps - 1) / kWarps, wave / 2 / pairs);
     S = std::max(S, S <= kMergeOneBatch ? std::min(single, kMergeOneBatch) : single);

@@ -158,8 +158,9 @@ struct DecodeArgs {
 constexpr int kAccStride = kMaxRatio * 128 + 32;  // floats per (b, kv) pair in DecodeArgs::acc
 
 cudaError_t launch_decode_scalar(const DecodeArgs& a, cudaStream_t st);
-// Fills S and the tile counts of `a` for the tensor-core kernel (S <= max_records; s_override > 0 forces S).
-void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_override);
+// Fills S, small and the tile counts of `a` for the tensor-core kernel (S <= max_records; s_override > 0 forces S).
+// may_be_small: the launch may take the form for small ones (DecodeArgs::small).
+void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_override, bool may_be_small);
 // Padded batch: shares one resident wave of CTAs out over the (b, kv) pairs in proportion to the tiles each
 // sequence still has to visit (rowinfo as in DecodeArgs, on the host).  Fills cta_map (room for
 // max_ctas_decode_mma(sm_count) entries) and pair_ctas (B * Hkv entries); returns the grid size and sets

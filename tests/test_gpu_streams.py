@@ -274,3 +274,21 @@ def test_small_launches_at_ordinary_lengths_are_reproducible(r, bits, group):
             cache.decode_attn(0, q, out)
         assert bool((outs == outs[0]).all()), n
         cache.close()
+
+
+def test_the_finer_split_of_small_launches_is_for_small_launches():
+    """Launches that may overlap, and timed ones, do not let the next one start early: they keep whole stages per warp."""
+    n, group = 1024, 32
+    k, v = synth.keys_values(9, 1, 2, n, D, "cuda")
+    splits = []
+    for flags in (0, LQ_FLAG_OVERLAP_DECODE):
+        cache = LogQuantCache(1, 1, 8, 2, 128, group, max_tokens=n + 8, flags=flags)
+        cache.append(0, k, v)
+        info = cache.info(0)
+        splits.append(info.n_splits)
+        if not flags:
+            cache.profile_enable()
+            splits.append(cache.info(0).n_splits)
+        cache.close()
+    tiles_fp, tiles_quant = -(-info.n_fp // 16), info.n_quant // group
+    assert splits == [-(-(tiles_fp + tiles_quant) // 4)] + 2 * [-(-(tiles_fp + tiles_quant // 2) // 4)]
