@@ -85,7 +85,12 @@ typedef enum {
  *     which is what frameworks issue by default): then q, k and v are complete before the decode launch starts.
  *     (A launch whose layer got a row from an earlier fused lq_append_decode_attn launch overlaps only once that
  *     launch is known to be complete, which the library derives from the launches enqueued since.)
- *     Without the flag every launch waits for its predecessor before it reads anything. */
+ *     Without the flag a launch waits for its predecessor before it reads anything -- except, on the tensor-core
+ *     kernel, a launch that leaves at least half of the GPU's slots for its CTAs empty (one or few sequences): when
+ *     the cache's previous call was a decode call on the same stream (both eager, or both in one capture) whose
+ *     launch appended no row to this layer, it fetches the first tiles of its layer's stores before it waits.
+ *     Everything that can have written those has finished by then; q, k, v and the workspace are touched only
+ *     after the wait, so no promise is asked of the caller. */
 #define LQ_FLAG_OVERLAP_DECODE 1
 
 typedef struct {

@@ -101,7 +101,8 @@ __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w &
 
 // Code i of either half of a word, masked in place, is the fp32 subnormal code * 2^(BITS i - 149): no conversion.  One
 // exact multiplication by 2^(127 - BITS i) turns it into code * 2^-22, for which x^ * 2^-22 = fma(., scale, zero * 2^-22)
-// rounds exactly as fma(code, scale, zero) does.
+// rounds exactly as fma(code, scale, zero) does, down to |x^| of about 2^-104, where the scaled result becomes subnormal
+// (its error is then at most 2^-128 in units of x^).
 constexpr float kCodeUnit = 0x1p-22f;
 template <int BITS>
 __device__ __forceinline__ uint64_t code_pair(uint32_t w, uint32_t whi, int i) {

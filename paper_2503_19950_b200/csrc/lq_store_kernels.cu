@@ -662,7 +662,7 @@ cudaError_t launch_ingest(const CacheView& cv, int layer, const void* k, const v
 }
 
 // ---------------------------------------------------------------------------------------
-// Blocks of a new cache (launch latency: seventeen memset calls took 70 us of the host's time, this one 4).
+// Blocks of a new cache (launch latency: fifteen memset calls took 70 us of the host's time, this one 4).
 // ---------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) lq_init_blocks_kernel(BlockInit b) {
   if (static_cast<int>(blockIdx.x) < b.n_guards) b.guard[blockIdx.x][threadIdx.x] = static_cast<uint8_t>(kGuardPattern);
