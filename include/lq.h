@@ -135,7 +135,8 @@ typedef struct {
   int32_t n_ctas;              /* CTAs of its attention kernel (tensor-core kernel; else 0)      */
   int64_t n_kernel_launches;   /* kernels this cache has launched so far (all layers)            */
   int32_t n_ctas_overlapped;   /* CTAs of an attention launch that overlaps the launch before it
-                                  (LQ_FLAG_OVERLAP_DECODE: a third of the resident wave; else 0)  */
+                                  (LQ_FLAG_OVERLAP_DECODE: a third of the resident wave, half of it above
+                                  256 MB per launch, at least one per pair; else 0)                */
   int32_t n_launches_overlapped; /* attention launches of this cache so far (all layers) that did overlap the
                                     launch before them                                               */
 } lq_info_t;

@@ -505,7 +505,7 @@ lq_status_t upload_masks(lq_cache* c, int layer, cudaStream_t st) {
     a.n_quant = L.n_quant;
     c->pad_grid[layer] = plan_decode_mma_padded(a, c->sm_count, c->max_splits, rowinfo, cta_map, pair_ctas,
                                                 &c->pad_stride[layer]);
-    // second plan, behind the first: a third of the wave for launches that overlap (LQ_FLAG_OVERLAP_DECODE)
+    // second plan, behind the first: a part of the wave for launches that overlap (LQ_FLAG_OVERLAP_DECODE)
     int32_t* pair_ctas_ov = cta_map + c->map_words;
     c->pad_grid_ov[layer] = plan_decode_mma_padded(a, c->sm_count, c->max_splits, rowinfo, pair_ctas_ov + B * c->cfg.n_kv_heads,
                                                    pair_ctas_ov, &c->pad_stride_ov[layer], true);
@@ -1378,7 +1378,7 @@ lq_status_t lq_cache_info(const lq_cache_t* c, int32_t layer, lq_info_t* info) {
     a.cv = c->cv;
     a.n_fp = L.n_fp;
     a.n_quant = L.n_quant;
-    a.early = 0;  // the plan of a launch that does not overlap (an overlapped one uses a third of these CTAs)
+    a.early = 0;  // the plan of a launch that does not overlap (an overlapped one uses a part of these CTAs)
     plan_decode_mma(a, c->sm_count, c->max_splits, c->cfg.n_splits, may_be_small(c));
     info->n_splits = a.S - 1;
     info->n_ctas = (a.S - 1) * c->cfg.batch * c->cfg.n_kv_heads + a.n_extra;

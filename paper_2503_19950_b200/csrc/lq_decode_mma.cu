@@ -53,7 +53,14 @@ __host__ __device__ constexpr int n_stages(int) { return 2; }
 __host__ __device__ constexpr int warp_stage_bytes(int G, int PL = 1) { return n_stages(G) * stage_bytes(G, PL); }
 constexpr int kWarpStageBytes = warp_stage_bytes(32);
 constexpr int kMaxStages = 3;
-constexpr int kOverlapDepth = 3;  // consecutive overlapped launches that share the SMs (plan_decode_mma)
+// Consecutive overlapped launches that share the SMs, by the bytes that a launch reads (DecodeArgs::early): each takes a third of
+// the slots with CTAs three times as long (at least one CTA per pair), so that every slot stays busy and the fixed costs of a
+// CTA (start-up, merge, ticket: 4 - 5 us) are paid once per three times the bytes (1/4 worse; 8k workload 15.4 -> 14.4 us per
+// launch).  With half of the slots the last launch of a series, which has nobody to share the SMs with, is over sooner (four
+// layers and a wait behind them, 97 to 394 MB per launch: 6 to 14 % less), but the fixed costs weigh more (among other
+// passes, up to four heads: +1 % at 97 MB, +0.4 to 0.9 % at 130 to 202 MB).  At 274 to 394 MB that is gone (-0.2 to +0.6 %).
+// Padded batches of 295 to 413 MB: 0 to 19 % less among other passes, -19 to +2 % with a wait behind them.
+__host__ constexpr int overlap_depth(int64_t bytes) { return bytes > (256LL << 20) ? 2 : 3; }
 constexpr int kCtasPerSm = 4;  // at 128 registers and 51 KB of shared memory; 3 and 5 both measured slower
 // More than four query heads per KV head need 168 registers (at 128 they spill: 16.4 instead of 14.5 us per layer on the
 // GQA-7 workload); the 9 KB stages of 4-bit codes at G = 64 leave shared memory for three CTAs as well, and these then take
@@ -66,8 +73,8 @@ constexpr int kSpinLimit = 1 << 22;
 // cost of one fp tile (16 bf16 tokens, two loads) in eighths of a quant tile: 4 to 12 measured alike,
 // 2 and 16 slower
 constexpr int kFpCost8 = 8;
-// (with two column blocks -- five to eight query heads per KV head -- a quant tile costs more and the bf16 tile
-// relatively less: 4, measured 2.5 % better than 8 on the GQA-7 workload)
+// (with five to eight query heads per KV head a quant tile costs more and the bf16 tile relatively less: 4, measured 2.5 %
+// better than 8 on the GQA-7 workload with an earlier form of the kernel, not since)
 __host__ __device__ constexpr int fp_cost8(int ncb) { return ncb == 2 ? 4 : kFpCost8; }
 
 // ---- PTX wrappers ----------------------------------------------------------------------
@@ -194,7 +201,8 @@ __device__ __forceinline__ uint32_t ext_f16(uint32_t w, uint32_t w10) {
   return I < 5 ? (w & (0x00030003u << (2 * I))) : (w10 & (0x00030003u << (2 * (I - 5))));
 }
 
-// NCB = number of column blocks of 4 heads.  NCB == 1: p.v columns are (hi, lo) per head and the
+// NCB = 1: up to four query heads per KV head, NCB = 2: five to eight (each lane then keeps scores, maximum and denominator
+// of two heads).  NCB == 1: p.v columns are (hi, lo) per head and the
 // probabilities carry a factor 2^64 (kPExp) so that products with bf16 subnormal codes stay normal.
 // NCB == 2: the probabilities (at most 2^8 because the reference maximum moves lazily) carry 2^-8, so
 // that p * s_v fits fp16 for every value scale fp16 itself can hold.
@@ -1258,19 +1266,11 @@ void plan_decode_mma(DecodeArgs& a, int sm_count, int max_records, int s_overrid
   const int items = a.tiles_fp + a.tiles_quant / (stage_bytes(a.cv.G, a.cv.planes) / quant_tile_bytes(a.cv.G, a.cv.planes));
   // at most one resident wave of CTAs in total: a CTA that had to wait for a free slot would start
   // when the others finish, and its pair's merge would wait for it
-  // the two-column-block variant needs more registers, the 9 KB stages of 4-bit codes at G = 64 more shared memory
   const int n_ctas_sm = ctas_per_sm(r <= 4 ? 1 : 2, a.cv.G, a.cv.planes);
-  // A serialised launch fills exactly one resident wave.  An overlapped launch (DecodeArgs::early) takes a third of
-  // the slots with CTAs three times as long (at least one CTA per pair): three consecutive launches then share the
-  // SMs, every slot stays busy, and the fixed costs of a CTA (start-up, merge, ticket: 4 - 5 us) are paid once per
-  // three times the bytes (measured: 1/2 and 1/3 alike, 1/4 worse; 8k workload 15.4 -> 14.4 us per launch).
-  // Above 256 MB per launch half of the slots do as well: the fixed costs no longer count, and the last launch of a series, which
-  // has nobody to share the SMs with, is over sooner (32 KV heads at 131072 tokens, four layers in a row and nothing behind them:
-  // 553 -> 484 us, among other passes 411 us either way; 47 to 116 MB per launch lose 1 to 7 %).
+  // a serialised launch fills exactly one resident wave, an overlapped one (DecodeArgs::early) its share of it
   const int64_t bytes = static_cast<int64_t>(pairs) * (static_cast<int64_t>(a.tiles_fp) * kFpTileBytes +
                                                        static_cast<int64_t>(a.tiles_quant) * quant_tile_bytes(a.cv.G, a.cv.planes));
-  const int depth = bytes > (256LL << 20) ? 2 : kOverlapDepth;
-  const int wave = a.early ? std::max(pairs, n_ctas_sm * sm_count / depth) : n_ctas_sm * sm_count;
+  const int wave = a.early ? std::max(pairs, n_ctas_sm * sm_count / overlap_depth(bytes)) : n_ctas_sm * sm_count;
   int S = s_override > 0 ? s_override : wave / pairs;
   S = std::min(S, (items + kWarps - 1) / kWarps);  // at least one item per warp
   // A serialised launch that leaves half of the slots empty is nothing but latency.  Its warps then take single tiles, up to
@@ -1310,18 +1310,19 @@ int plan_decode_mma_padded(const DecodeArgs& a, int sm_count, int max_records, c
   const int tiles_quant = static_cast<int>(a.n_quant / a.cv.G);
   const int tps = stage_bytes(a.cv.G, a.cv.planes) / quant_tile_bytes(a.cv.G, a.cv.planes);
   const int slots = ctas_per_sm(r <= 4 ? 1 : 2, a.cv.G, a.cv.planes) * sm_count;
-  const int wave = overlapped ? std::max(pairs, slots / kOverlapDepth) : slots;  // as in plan_decode_mma
   const int cap_records = std::max(1, std::min(max_records, kMergeMax / r));
   std::vector<int64_t> work(pairs);
   std::vector<int> cap(pairs);
-  int64_t total = 0;
+  int64_t total = 0, bytes = static_cast<int64_t>(pairs) * tiles_fp * kFpTileBytes;
   for (int p = 0; p < pairs; ++p) {
     const int tq = std::max(0, tiles_quant - rowinfo_host[4 * (p / a.cv.Hkv) + 0]);
     work[p] = static_cast<int64_t>(tiles_fp) * fp_cost8(r <= 4 ? 1 : 2) + 8LL * tq;  // the kernel's cost line
     const int items = tiles_fp + tq / tps;
     cap[p] = std::max(1, std::min(cap_records, items / kWarps));  // at least one item per warp
     total += work[p];
+    bytes += static_cast<int64_t>(tq) * quant_tile_bytes(a.cv.G, a.cv.planes);
   }
+  const int wave = overlapped ? std::max(pairs, slots / overlap_depth(bytes)) : slots;  // as in plan_decode_mma
   // largest-remainder shares of one wave, clipped to the caps
   int given = 0;
   std::vector<std::pair<int64_t, int>> rest(pairs);

@@ -321,3 +321,38 @@ def test_long_run_of_overlapped_fused_steps_over_32_layers():
     cache.close()
     for oc in ocs.values():
         oc.close()
+
+
+@pytest.mark.parametrize("ctx,padded,depth", [(24576, False, 3), (49152, False, 2), (65536, True, 2)])
+def test_overlapped_launches_on_both_sides_of_256_mb(ctx, padded, depth):
+    """Launches of 151, 302 and (left-padded) 315 MB: the share of the resident wave that they take, and the same attention
+    from launches that overlap and from launches that are timed, hence serialised.  Either carries its probabilities in two
+    bf16 parts, which leave out at most 2^-17 of each, and the values as zero + code * scale, |zero| <= max|v| and
+    code * scale <= 2 max|v|: the two differ by at most 2 * 2^-17 * 3 max|v|."""
+    from paper_2503_19950_b200 import LQ_FLAG_OVERLAP_DECODE
+    L, B, H = 3, 2, 32
+    cache = LogQuantCache(L, B, H, H, 256, 32, max_tokens=ctx + 8, flags=LQ_FLAG_OVERLAP_DECODE)
+    gen = torch.Generator(device="cuda").manual_seed(ctx)
+    vmax = 0.0
+    for layer in range(L):
+        k, v = (torch.randn(B, H, ctx, D, generator=gen, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+        cache.append(layer, k, v)
+        vmax = max(vmax, float(v.max()), -float(v.min()))
+    slots = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert cache.info(0).n_ctas_overlapped == slots // depth
+    if padded:
+        cache.set_padding([0, ctx * 7 // 16])
+    q = torch.randn(L, B, H, D, generator=gen, device="cuda", dtype=torch.bfloat16)
+    out = torch.empty(2, L, B, H, D, device="cuda")
+    overlapped = []
+    for form in (0, 0, 1):   # (a first pass uploads the masks of every layer)
+        if form:
+            cache.profile_enable()
+        for layer in range(L):
+            cache.decode_attn(layer, q[layer], out[form, layer])
+        overlapped.append(cache.info(0).n_launches_overlapped)
+    torch.cuda.synchronize()
+    assert overlapped[1] - overlapped[0] == L and overlapped[2] == overlapped[1]
+    assert float((out[0] - out[1]).abs().max()) <= 2 * 2.0 ** -17 * 3 * vmax
+    assert cache.kernel_status() == 0
+    cache.close()
