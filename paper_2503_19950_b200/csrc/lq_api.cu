@@ -100,7 +100,7 @@ struct lq_cache {
   uint32_t* masks = nullptr;
   int fp_words = 0, q_words = 0, map_words = 0;
   int64_t mask_layer_words = 0;
-  std::vector<uint32_t> mask_host;
+  std::vector<std::vector<uint32_t>> mask_host;  // per layer: a captured upload reads it when the graph runs
   std::vector<int> pad_grid, pad_stride;  // per layer: CTAs and record stride of the padded tensor-core launch
   std::vector<int> pad_grid_ov, pad_stride_ov;  // the same for a launch that overlaps the one before it
   // optional timing of the split-K attention kernel
@@ -463,9 +463,10 @@ bool use_umma(const lq_cache* c) { return c->cfg.kernel == LQ_KERNEL_UMMA && !c-
 lq_status_t upload_masks(lq_cache* c, int layer, cudaStream_t st) {
   const LayerState& L = c->layers[layer];
   const int B = c->cfg.batch, G = c->cfg.group;
-  c->mask_host.assign(static_cast<size_t>(c->mask_layer_words), 0u);
-  int32_t* rowinfo = reinterpret_cast<int32_t*>(c->mask_host.data());
-  uint32_t* fpm = c->mask_host.data() + 4 * B;
+  std::vector<uint32_t>& host = c->mask_host[layer];
+  host.assign(static_cast<size_t>(c->mask_layer_words), 0u);
+  int32_t* rowinfo = reinterpret_cast<int32_t*>(host.data());
+  uint32_t* fpm = host.data() + 4 * B;
   uint32_t* qm = fpm + static_cast<size_t>(c->fp_words) * B;
   const int64_t tiles = L.n_quant / G;
   for (int b = 0; b < B; ++b) {
@@ -510,10 +511,10 @@ lq_status_t upload_masks(lq_cache* c, int layer, cudaStream_t st) {
     c->pad_grid_ov[layer] = plan_decode_mma_padded(a, c->sm_count, c->max_splits, rowinfo, pair_ctas_ov + B * c->cfg.n_kv_heads,
                                                    pair_ctas_ov, &c->pad_stride_ov[layer], true);
   }
-  // pageable source: staged by the runtime before the call returns
+  // pageable source: staged by the runtime before the call returns, unless the stream is being captured
   c->last_decode_layer = -1;
-  cudaError_t e = cudaMemcpyAsync(c->masks + layer * c->mask_layer_words, c->mask_host.data(),
-                                  c->mask_host.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, st);
+  cudaError_t e = cudaMemcpyAsync(c->masks + layer * c->mask_layer_words, host.data(), host.size() * sizeof(uint32_t),
+                                  cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return cuda_fail(c, e, "padding mask upload");
   c->mask_dirty[layer] = 0;
   return LQ_OK;
@@ -1047,6 +1048,7 @@ lq_status_t lq_set_padding(lq_cache_t* c, const int32_t* pad_host) {
   c->has_pad = false;
   for (int b = 0; b < B; ++b) c->has_pad |= pad_host[b] > 0;
   c->mask_dirty.assign(c->cfg.n_layers, 1);
+  c->mask_host.resize(c->cfg.n_layers);
   c->pad_grid.assign(c->cfg.n_layers, 0);
   c->pad_stride.assign(c->cfg.n_layers, 1);
   c->pad_grid_ov.assign(c->cfg.n_layers, 0);

@@ -146,6 +146,34 @@ def test_prompts_ingested_under_capture(window, group):
     cache.close()
 
 
+def test_padding_masks_uploaded_under_capture():
+    """Two layers in different states whose masks are made in one capture: every replay finds its own layer's masks."""
+    lengths, pad = (150, 217), 40
+    cache = LogQuantCache(2, 2, HQ, HKV, W, G, max_tokens=256)
+    oracles = []
+    for layer, n in enumerate(lengths):
+        k, v = synth.keys_values(50 + layer, 2, HKV, n, D, "cuda")
+        cache.append(layer, k, v)
+        oracles.append(oracle.OracleCache(2, HQ, HKV, D, W, G))
+        oracles[-1].append(synth.bf16_bits(k), synth.bf16_bits(v))
+    q, out = synth.queries(51, 2, HQ, D, 0, "cuda"), torch.full((2, 2, HQ, D), float("nan"), device="cuda")
+    cache.set_padding([0, pad])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for layer in range(2):
+            cache.decode_attn(layer, q, out[layer])
+    for _ in range(2):
+        out.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        for layer in range(2):
+            ref = oracles[layer].attention_subset(synth.bf16_bits(q), 1 / np.sqrt(D), pad=[0, pad])
+            assert np.abs(out[layer].cpu().numpy() - ref).max() <= attn_tolerance(ref)
+    assert cache.kernel_status() == 0
+    cache.close()
+
+
 def _two_layers(flags=0):
     """A cache of two small layers with a few steps behind them, and the calls of further steps."""
     cache = LogQuantCache(2, B, HQ, HKV, W, G, max_tokens=256, flags=flags)
@@ -292,3 +320,46 @@ def test_the_finer_split_of_small_launches_is_for_small_launches():
         cache.close()
     tiles_fp, tiles_quant = -(-info.n_fp // 16), info.n_quant // group
     assert splits == [-(-(tiles_fp + tiles_quant) // 4)] + 2 * [-(-(tiles_fp + tiles_quant // 2) // 4)]
+
+
+@pytest.mark.parametrize("bits,group,n,heads", [(2, 32, 1200, (8, 2)), (2, 32, 6000, (4, 1)), (2, 64, 5000, (7, 1)), (4, 32, 3000, (8, 2)),
+                                                (4, 64, 4000, (4, 4))])
+@pytest.mark.parametrize("host", [False, True])
+def test_small_launches_that_fetch_early_in_every_form(bits, group, n, heads, host):
+    """Steps of two layers in turn, device-resident or with the rows, queries and results in pinned host memory, all of them
+    behind a launch of the other layer: ordered merges and (more than 12 CTAs per pair) sums on arrival, both group sizes
+    and widths, up to four and more heads per KV head."""
+    hq, hkv = heads
+    steps = 5
+    cache = LogQuantCache(2, B, hq, hkv, 64, group, max_tokens=n + steps + 8, bits=bits)
+    oracles, rows = [], []
+    for layer in range(2):
+        k, v = synth.keys_values(30 + layer, B, hkv, n + steps, D, "cuda")
+        cache.append(layer, k[:, :, :n].contiguous(), v[:, :, :n].contiguous())
+        oracles.append(oracle.OracleCache(B, hq, hkv, D, 64, group, bits=bits))
+        oracles[-1].append(synth.bf16_bits(k[:, :, :n]), synth.bf16_bits(v[:, :, :n]))
+        rows.append([tuple(x[:, :, n + s:n + s + 1].contiguous() for x in (k, v)) for s in range(steps)])
+    assert (cache.info(0).n_splits > 12) == (n >= 3000)
+    qs = [[synth.queries(31 + layer, B, hq, D, s, "cuda") for layer in range(2)] for s in range(steps)]
+    outs = torch.full((steps, 2, B, hq, D), float("nan"), device="cuda")
+    if host:
+        pin = lambda x: torch.empty(x.shape, dtype=x.dtype, pin_memory=True).copy_(x)
+        rows = [[tuple(pin(x) for x in row) for row in layer] for layer in rows]
+        qs, outs = [[pin(q) for q in step] for step in qs], pin(outs)
+    torch.cuda.synchronize()
+    for s in range(steps):
+        for layer in range(2):
+            if host:
+                cache.decode_step_host(layer, *rows[layer][s], qs[s][layer], outs[s, layer], sync=False)
+            else:
+                cache.append_decode_attn(layer, *rows[layer][s], qs[s][layer], outs[s, layer])
+    torch.cuda.synchronize()
+    assert cache.debug_launches_prefetched() == 2 * steps - 1   # no overflow falls into these steps
+    for s in range(steps):
+        for layer in range(2):
+            oracles[layer].append(*(synth.bf16_bits(x) for x in rows[layer][s]))
+            _check_attention(oracles[layer], qs[s][layer], outs[s, layer])
+    for layer in range(2):
+        assert_images_equal(cache.export(layer), oracles[layer].export())
+    assert cache.kernel_status() == 0
+    cache.close()
