@@ -108,6 +108,50 @@ def test_random_images_against_the_same_attention_in_64_bits(r, G, bits, n_fp, n
     assert float((out.double() - want).norm() / want.norm()) < 1e-5
 
 
+@pytest.mark.parametrize("r,G,bits,n_fp,n_quant,off", [(4, 32, 2, 40, 32 * 3, 0), (4, 32, 2, 385, 32 * 60, 0), (7, 64, 4, 200, 64 * 20, 0),
+                                                       (2, 32, 4, 100, 32 * 30, 1)])
+def test_captured_calls_give_what_eager_calls_give(r, G, bits, n_fp, n_quant, off):
+    """One split and several, wide and byte-wise fetches, two calls in a row in one graph (the second finds the first one's
+    partials in the scratch), replayed on other inputs than those of the capture."""
+    build.build()
+    B, H, gen = 2, 2, torch.Generator(device="cuda").manual_seed(n_quant)
+
+    def place(x):  # a copy of x that starts `off` elements behind a 16-byte boundary
+        buf = torch.empty(x.numel() + 16, dtype=x.dtype, device="cuda")
+        y = buf[off:off + x.numel()].view(x.shape)
+        y.copy_(x)
+        return y
+
+    def bf16(*shape):
+        return place(torch.randn(*shape, generator=gen, device="cuda", dtype=torch.bfloat16).view(torch.int16))
+
+    def codes():
+        return place(torch.randint(0, 256, (B, H, n_quant, D * bits // 8), generator=gen, device="cuda", dtype=torch.uint8))
+
+    image = dict(fp_k=bf16(B, H, n_fp, D), fp_v=bf16(B, H, n_fp, D), k_codes=codes(), v_codes=codes(),
+                 k_scale=bf16(B, H, n_quant // G, D), k_zero=bf16(B, H, n_quant // G, D),
+                 v_scale=bf16(B, H, n_quant, D // G), v_zero=bf16(B, H, n_quant, D // G))
+    q = torch.randn(2, B, H * r, D, generator=gen, device="cuda", dtype=torch.bfloat16)
+    out = torch.empty(2, B, H * r, D, device="cuda")
+
+    def calls():
+        for i in range(2):
+            assert decode_attn_image_static(image, H * r, G, q[i], out[i], bits=bits) == binding.LQ_OK
+
+    calls()   # (the first call on a device comes before any capture)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        calls()
+    q.copy_(torch.randn(q.shape, generator=gen, device="cuda", dtype=torch.bfloat16))
+    calls()
+    want = out.clone()
+    out.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert bool(want.isfinite().all()) and torch.equal(out, want)
+
+
 def _empty_image(B):
     z16 = torch.zeros(1, dtype=torch.int16, device="cuda")
     return dict(fp_k=torch.zeros(B, 1, 1, 128, dtype=torch.int16, device="cuda"),
