@@ -181,7 +181,7 @@ class LogQuantCache:
         # the calls of a decode step, bound once
         self._append_decode_attn, self._decode_attn = self._lib.lq_append_decode_attn, self._lib.lq_decode_attn
         self._decode_step_host = self._lib.lq_decode_step_host
-        self._blocks = {}
+        blocks = self._blocks = {}  # (the callbacks hold this, not self: the cache is freed with its last reference)
         LogQuantCache.live.add(self)
         alloc_cb, free_cb = ALLOC_FN(0), FREE_FN(0)
         pool = None  # handle of the stream whose pool the blocks come from
@@ -202,11 +202,11 @@ class LogQuantCache:
                             t = torch.empty(nbytes, dtype=torch.uint8, device=where)
                 except RuntimeError:
                     return 0
-                self._blocks[t.data_ptr()] = t
+                blocks[t.data_ptr()] = t
                 return t.data_ptr()
 
             def _free(ptr, _ctx):
-                self._blocks.pop(ptr, None)
+                blocks.pop(ptr, None)
 
             alloc_cb, free_cb = ALLOC_FN(_alloc), FREE_FN(_free)
         elif allocator is not None:

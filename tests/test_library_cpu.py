@@ -1,7 +1,9 @@
 """CPU-only checks of the CUDA library: it loads, exports what include/lq.h declares, validates
 arguments, and its host-side mirror of Algorithm 1 agrees with the oracle (bookkeeping-only mode)."""
+import gc
 import os
 import re
+import weakref
 
 import numpy as np
 import pytest
@@ -27,6 +29,19 @@ def test_library_exports_every_declared_symbol():
     for name in declared:
         assert hasattr(lib, name), name
     assert sorted(binding.SYMBOLS) == declared
+
+
+@pytest.mark.parametrize("allocator", [None, "torch"])
+def test_a_cache_is_freed_with_its_last_reference(allocator):
+    """Its device memory does not wait for a run of the cycle collector."""
+    cache = _dry(W=128, G=32, allocator=allocator)
+    gone = weakref.ref(cache)
+    gc.disable()
+    try:
+        del cache
+        assert gone() is None
+    finally:
+        gc.enable()
 
 
 def test_status_strings():
