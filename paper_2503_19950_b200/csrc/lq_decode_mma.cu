@@ -427,9 +427,10 @@ __device__ __forceinline__ void patch_new_row(uint32_t half_tile_smem, uint8_t* 
 // ---- one quant tile: one key group of G tokens ---------------------------------------------
 // PL = 2-bit planes per code.  A 4-bit code is 4 * (high plane) + (low plane).  In q.k, up to 4 heads and G = 32, the low
 // plane meets a quarter of q * s and the sum counts four times: the key scale is folded in once for both planes
-// (22.2 -> 21.6 us per layer, B = 8, 32/8 heads, 8192 tokens).  With more heads, where q * s takes two operands, and at
-// G = 64 that costs registers (27.2 -> 28.7 us, 64/8 heads; 19.9 -> 20.0 us): the high plane goes first and its accumulators
-// are multiplied by 4 before the low plane is added.  In p.v the high plane meets p * s_v * 4 (all exact).
+// (22.2 -> 21.6 us per layer, B = 8, 32/8 heads, 8192 tokens; 24.4 -> 24.0 once the power cap has set in).  With more heads,
+// where q * s takes two operands, and at G = 64 that costs registers (27.2 -> 28.7 us, 64/8 heads; 19.9 -> 20.0 us): the high
+// plane goes first and its accumulators are multiplied by 4 before the low plane is added.  In p.v the high plane meets
+// p * s_v * 4 (all exact).
 template <int G, int NCB, int PL>
 __host__ __device__ constexpr int planes_together() { return G == 32 && NCB == 1 ? PL : 1; }
 // pad0/pad1: bit i set = token i (pad0) or 32 + i (pad1) of the tile is padding (left out); not all of them are
